@@ -34,6 +34,7 @@
 #include <vector>
 
 #include "vq_async.cuh"
+#include "vq_energy_mma.cuh"
 #include "vq_internal.cuh"
 
 namespace vq {
@@ -472,7 +473,8 @@ BatchKernel batch_kernel(int prec, int terms, int stages, int method) {
 // Exact energies of x_r = [S_r > 0] in the same fixed point as a single
 // context's readout: parts[g][r] = sum over the 64 rows of tile g of
 // x_ri (dfix_i + sum_{j != i} round(Q_ij 2^shift) x_rj), Q as given. A block
-// takes one (instance, 64-row tile, 32-replica tile) item of the work list.
+// takes one (instance, 64-row tile, replica tile) item of the work list
+// (vq_energy_mma.cuh).
 struct ReadInst {
     const void* q;           // [n][n] Q as given (element type of the launch)
     const int64_t* dfix;     // [n]
@@ -481,63 +483,25 @@ struct ReadInst {
     uint8_t* x;              // [n] winner's vector
     int32_t n, shift;
 };
-template <typename QT>
-__global__ void __launch_bounds__(256) k_batch_energy(const ReadInst* __restrict__ insts,
-                                                      const int32_t* __restrict__ work, int32_t R) {
-    __shared__ int64_t qt[64][33];
-    __shared__ uint32_t xw[32];
-    __shared__ int64_t red[8][32];
+template <int TR, typename QT>
+__global__ void __launch_bounds__(4 * TR, 512 / (4 * TR)) k_batch_energy(const ReadInst* __restrict__ insts,
+                                                                         const int32_t* __restrict__ work,
+                                                                         int32_t R) {
+    __shared__ emma::Smem<TR> sm;
     const int32_t m = work[2 * blockIdx.x], local = work[2 * blockIdx.x + 1];
     const ReadInst in = insts[m];
-    const int32_t n = in.n;
-    const int32_t tiles = (n + 63) / 64;
+    const int32_t tiles = (in.n + emma::TI - 1) / emma::TI;
     const int32_t tile = local % tiles, rt = local / tiles;
-    const QT* Q = static_cast<const QT*>(in.q);
-    const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
-    const int32_t r = rt * 32 + lane;
-    const int64_t i0 = (int64_t)tile * 64;
-    int64_t row[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) row[q] = 0;
-    for (int64_t j0 = 0; j0 < n; j0 += 32) {
-        __syncthreads();
-        for (int e = threadIdx.x; e < 64 * 32; e += 256) {
-            const int ii = e / 32, jj = e % 32;
-            const int64_t gi = i0 + ii, gj = j0 + jj;
-            qt[ii][jj] = (gi < n && gj < n && gi != gj) ? vqd::qfix<QT>(Q[gi * n + gj], in.shift) : 0;
-        }
-        if (g == 0) {
-            uint32_t w = 0;
-            if (r < R)
-                for (int jj = 0; jj < 32; ++jj) {
-                    const int64_t gj = j0 + jj;
-                    if (gj < n && in.S[(int64_t)r * n + gj] > 0.0f) w |= 1u << jj;
-                }
-            xw[lane] = w;
-        }
-        __syncthreads();
-        const uint32_t w = xw[lane];
-#pragma unroll 4
-        for (int jj = 0; jj < 32; ++jj) {
-            const bool on = (w >> jj) & 1u;
-#pragma unroll
-            for (int q = 0; q < 8; ++q) row[q] += on ? qt[g * 8 + q][jj] : 0;
-        }
-    }
-    int64_t part = 0;
-    if (r < R) {
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int64_t gi = i0 + g * 8 + q;
-            if (gi < n && in.S[(int64_t)r * n + gi] > 0.0f) part += __ldg(in.dfix + gi) + row[q];
-        }
-    }
-    red[g][lane] = part;
-    __syncthreads();
-    if (g == 0 && r < R) {
-        int64_t tot = 0;
-        for (int q = 0; q < 8; ++q) tot += red[q][lane];
-        in.parts[(int64_t)tile * R + r] = tot;
+    emma::energy_tile<TR, QT, float>(sm, R, in.n, static_cast<const QT*>(in.q), in.shift, in.dfix, in.S,
+                                     (int64_t)tile * emma::TI, (int64_t)rt * TR, in.parts + (int64_t)tile * R);
+}
+template <int TR>
+void launch_batch_energy(int type, unsigned blocks, cudaStream_t st, const ReadInst* rd, const int32_t* wd, int32_t R) {
+    switch (type) {
+        case VELOXQ_I8: k_batch_energy<TR, int8_t><<<blocks, 4 * TR, 0, st>>>(rd, wd, R); break;
+        case VELOXQ_I32: k_batch_energy<TR, int32_t><<<blocks, 4 * TR, 0, st>>>(rd, wd, R); break;
+        case VELOXQ_F32: k_batch_energy<TR, float><<<blocks, 4 * TR, 0, st>>>(rd, wd, R); break;
+        default: k_batch_energy<TR, double><<<blocks, 4 * TR, 0, st>>>(rd, wd, R); break;
     }
 }
 
@@ -607,7 +571,8 @@ bool batch_supported(veloxq_ctx* const* ctxs, int32_t count, int32_t R, const Ru
 }
 
 // Runs the persistent batched kernel, then the exact final-readout energies and
-// the argmin of every instance. stages: 4 (two CTAs per SM) or 6 (one).
+// the argmin of every instance; without `graph` only the kernel, timed (the
+// autotuner's probes). stages: 4 (two CTAs per SM) or 6 (one).
 int batch_run(veloxq_ctx* const* ctxs, int32_t count, int32_t R, const RunParams& p, uint64_t seed, cudaStream_t st,
               int stages, int split, DevBuf& work, int64_t* d_best_all, int* d_err, float* ms_main,
               int64_t* launches, BatchGraph* graph) {
@@ -705,19 +670,20 @@ int batch_run(veloxq_ctx* const* ctxs, int32_t count, int32_t R, const RunParams
         begin.push_back((int32_t)order.size());
     }
     // the final readout's tables: one entry per instance, and per element type
-    // of Q a work list of (instance, 64-row tile, 32-replica tile) items
+    // of Q a work list of (instance, 64-row tile, replica tile) items
     std::vector<ReadInst> rd((size_t)count);
     std::vector<int32_t> rwork[4];
+    const int etr = emma::tile_replicas(R);
     for (int m = 0; m < count; ++m) {
         veloxq_ctx* c = ctxs[m];
-        const int tiles = (int)div_up(c->n, 64);
+        const int tiles = (int)div_up(c->n, emma::TI);
         VQ_TRY(c->ework.ensure(sizeof(int64_t) * (size_t)tiles * R));
         VQ_TRY(c->xout.ensure((size_t)c->n));
         rd[m] = ReadInst{c->qx.p, c->dfix.as<int64_t>(), c->s_a.as<float>(), c->ework.as<int64_t>(),
                          c->xout.as<uint8_t>(), (int32_t)c->n, c->energy_shift};
         const int t = (int)c->qx_type;
         if (t < 0 || t > 3) return fail(VELOXQ_EINVAL, "unknown coupling type");
-        for (int l = 0; l < tiles * (int)div_up(R, 32); ++l) {
+        for (int l = 0; l < tiles * (int)div_up(R, etr); ++l) {
             rwork[t].push_back(m);
             rwork[t].push_back(l);
         }
@@ -786,16 +752,13 @@ int batch_run(veloxq_ctx* const* ctxs, int32_t count, int32_t R, const RunParams
         fn<<<ctas, stages == 6 ? batch_threads<6>() : batch_threads<4>(), smem, st>>>(a);
         VQ_LAUNCH_CHECK("batch kernel");
         VQ_CUDA(cudaEventRecordWithFlags(e1, st, flags));
+        if (!graph) return VELOXQ_OK;   // a timing probe of the form: no readout
         for (int t = 0; t < 4; ++t) {
             const unsigned blocks = (unsigned)(rwork[t].size() / 2);
             if (!blocks) continue;
             const int32_t* wd = reinterpret_cast<const int32_t*>(wl[t]);
-            switch (t) {
-                case VELOXQ_I8: k_batch_energy<int8_t><<<blocks, 256, 0, st>>>(rdev, wd, R); break;
-                case VELOXQ_I32: k_batch_energy<int32_t><<<blocks, 256, 0, st>>>(rdev, wd, R); break;
-                case VELOXQ_F32: k_batch_energy<float><<<blocks, 256, 0, st>>>(rdev, wd, R); break;
-                default: k_batch_energy<double><<<blocks, 256, 0, st>>>(rdev, wd, R); break;
-            }
+            if (etr == emma::TR_WIDE) launch_batch_energy<emma::TR_WIDE>(t, blocks, st, rdev, wd, R);
+            else launch_batch_energy<emma::TR_NARROW>(t, blocks, st, rdev, wd, R);
         }
         k_batch_finish<<<(unsigned)count, 256, 0, st>>>(rdev, R, d_best_all);
         VQ_LAUNCH_CHECK("batch readout");

@@ -4,6 +4,7 @@
 // epilogue, and the exact readout energy in int64 fixed point.
 #include <algorithm>
 
+#include "vq_energy_mma.cuh"
 #include "vq_internal.cuh"
 
 namespace vq {
@@ -216,68 +217,17 @@ __global__ void __launch_bounds__(256) k_dense_finish(int32_t R, int32_t n, int 
 
 // Exact energy of x_r = [S_r > 0] (or of a caller batch of bytes), fixed
 // point: parts[g][r] = sum over the 64 rows of tile g of
-// x_ri (dfix_i + sum_{j != i} qfix(Q_ij) x_rj), Q as given.
-// Block: 32 replicas x 8 row groups; the Q tile is staged in shared memory
-// as int64 and broadcast to the 32 replica lanes.
-template <typename QT, bool FROM_BYTES>
-__global__ void __launch_bounds__(256) k_dense_energy(int64_t R, int32_t n, const QT* __restrict__ Q, int shift,
-                                                      const int64_t* __restrict__ dfix, const float* __restrict__ S,
-                                                      const uint8_t* __restrict__ X, int64_t* __restrict__ parts) {
-    __shared__ int64_t qt[64][33];
-    __shared__ uint32_t xw[32];
-    __shared__ int64_t red[8][32];
-    const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
-    const int64_t r = (int64_t)blockIdx.y * 32 + lane;
-    const int64_t i0 = (int64_t)blockIdx.x * 64;
-    int64_t row[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) row[q] = 0;
-    for (int64_t j0 = 0; j0 < n; j0 += 32) {
-        __syncthreads();
-        for (int e = threadIdx.x; e < 64 * 32; e += 256) {
-            const int ii = e / 32, jj = e % 32;
-            const int64_t gi = i0 + ii, gj = j0 + jj;
-            qt[ii][jj] = (gi < n && gj < n && gi != gj) ? vqd::qfix<QT>(Q[gi * n + gj], shift) : 0;
-        }
-        if (g == 0) {
-            // bit jj of xw[lane] = x[r][j0 + jj]
-            uint32_t w = 0;
-            if (r < R)
-                for (int jj = 0; jj < 32; ++jj) {
-                    const int64_t gj = j0 + jj;
-                    bool b = false;
-                    if (gj < n) b = FROM_BYTES ? X[r * n + gj] != 0 : S[r * n + gj] > 0.0f;
-                    w |= (uint32_t)b << jj;
-                }
-            xw[lane] = w;
-        }
-        __syncthreads();
-        const uint32_t w = xw[lane];
-#pragma unroll 4
-        for (int jj = 0; jj < 32; ++jj) {
-            const bool on = (w >> jj) & 1u;
-#pragma unroll
-            for (int q = 0; q < 8; ++q) row[q] += on ? qt[g * 8 + q][jj] : 0;
-        }
-    }
-    int64_t part = 0;
-    if (r < R) {
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int64_t gi = i0 + g * 8 + q;
-            if (gi < n) {
-                const bool xi = FROM_BYTES ? X[r * n + gi] != 0 : S[r * n + gi] > 0.0f;
-                if (xi) part += __ldg(dfix + gi) + row[q];
-            }
-        }
-    }
-    red[g][lane] = part;
-    __syncthreads();
-    if (g == 0 && r < R) {
-        int64_t tot = 0;
-        for (int q = 0; q < 8; ++q) tot += red[q][lane];
-        parts[(int64_t)blockIdx.x * R + r] = tot;
-    }
+// x_ri (dfix_i + sum_{j != i} qfix(Q_ij) x_rj), Q as given. One block per
+// tile of 64 rows and TR replicas (vq_energy_mma.cuh).
+template <int TR, typename QT, typename XT>
+__global__ void __launch_bounds__(4 * TR, 512 / (4 * TR)) k_dense_energy(int64_t R, int32_t n,
+                                                                         const QT* __restrict__ Q, int shift,
+                                                                         const int64_t* __restrict__ dfix,
+                                                                         const XT* __restrict__ x,
+                                                                         int64_t* __restrict__ parts) {
+    __shared__ emma::Smem<TR> sm;
+    emma::energy_tile<TR, QT, XT>(sm, R, n, Q, shift, dfix, x, (int64_t)blockIdx.x * emma::TI,
+                                  (int64_t)blockIdx.y * TR, parts + (int64_t)blockIdx.x * R);
 }
 
 // k-splits of the FP32 dense step: enough CTAs to fill the GPU when the
@@ -329,30 +279,35 @@ int launch_dense_step(veloxq_ctx* ctx, int32_t R, const float* S_cur, float* S_n
     return VELOXQ_OK;
 }
 
-template <bool FROM_BYTES>
-int launch_dense_energy(veloxq_ctx* ctx, int64_t R, const float* S, const uint8_t* X, int64_t* parts, int* nparts,
-                        bool allow_tc) {
+// The four element types Q can come in; x: float state or byte vectors.
+template <int TR, typename XT>
+void launch_energy_tiles(veloxq_ctx* ctx, int64_t R, const XT* x, int64_t* parts) {
     const int32_t n = (int32_t)ctx->n;
-    *nparts = (int)div_up(n, 64);
-    if (R == 0) return VELOXQ_OK;
-    if (allow_tc && tc_energy_ready(ctx, R)) return tc_energy(ctx, R, S, X, parts, nparts);
-    dim3 g((unsigned)div_up(n, 64), (unsigned)div_up(R, 32));
+    const dim3 g((unsigned)div_up(n, emma::TI), (unsigned)div_up(R, TR));
     const int sh = ctx->energy_shift;
     const int64_t* df = ctx->dfix.as<int64_t>();
+#define VQ_EN(QT) k_dense_energy<TR, QT, XT><<<g, 4 * TR, 0, ctx->stream>>>(R, n, ctx->qx.as<QT>(), sh, df, x, parts)
     switch (ctx->qx_type) {
-        case VELOXQ_I8:
-            k_dense_energy<int8_t, FROM_BYTES><<<g, 256, 0, ctx->stream>>>(R, n, ctx->qx.as<int8_t>(), sh, df, S, X, parts);
-            break;
-        case VELOXQ_I32:
-            k_dense_energy<int32_t, FROM_BYTES><<<g, 256, 0, ctx->stream>>>(R, n, ctx->qx.as<int32_t>(), sh, df, S, X, parts);
-            break;
-        case VELOXQ_F32:
-            k_dense_energy<float, FROM_BYTES><<<g, 256, 0, ctx->stream>>>(R, n, ctx->qx.as<float>(), sh, df, S, X, parts);
-            break;
-        case VELOXQ_F64:
-            k_dense_energy<double, FROM_BYTES><<<g, 256, 0, ctx->stream>>>(R, n, ctx->qx.as<double>(), sh, df, S, X, parts);
-            break;
+        case VELOXQ_I8: VQ_EN(int8_t); break;
+        case VELOXQ_I32: VQ_EN(int32_t); break;
+        case VELOXQ_F32: VQ_EN(float); break;
+        case VELOXQ_F64: VQ_EN(double); break;
     }
+#undef VQ_EN
+}
+template <typename XT>
+void launch_energy_tiles(veloxq_ctx* ctx, int64_t R, const XT* x, int64_t* parts) {
+    if (emma::tile_replicas(R) == emma::TR_WIDE) launch_energy_tiles<emma::TR_WIDE>(ctx, R, x, parts);
+    else launch_energy_tiles<emma::TR_NARROW>(ctx, R, x, parts);
+}
+
+int launch_dense_energy(veloxq_ctx* ctx, int64_t R, const float* S, const uint8_t* X, int64_t* parts, int* nparts,
+                        bool allow_tc) {
+    *nparts = (int)div_up(ctx->n, emma::TI);
+    if (R == 0) return VELOXQ_OK;
+    if (allow_tc && tc_energy_ready(ctx, R)) return tc_energy(ctx, R, S, X, parts, nparts);
+    if (X) launch_energy_tiles(ctx, R, X, parts);
+    else launch_energy_tiles(ctx, R, S, parts);
     VQ_LAUNCH_CHECK("dense_energy");
     return VELOXQ_OK;
 }
@@ -378,11 +333,11 @@ int dense_field(veloxq_ctx* ctx, int32_t R, const float* S, float* F) {
 // allow_tc: the tensor-core form when tc_energy_prepare has sized it for R
 // replicas (the caller then checks ctx->errw)
 int dense_energy(veloxq_ctx* ctx, int32_t R, const float* S, int64_t* parts, int* nparts, bool allow_tc) {
-    return launch_dense_energy<false>(ctx, R, S, nullptr, parts, nparts, allow_tc);
+    return launch_dense_energy(ctx, R, S, nullptr, parts, nparts, allow_tc);
 }
 
 int dense_energy_x(veloxq_ctx* ctx, int64_t B, const uint8_t* X, int64_t* parts, int* nparts, bool allow_tc) {
-    return launch_dense_energy<true>(ctx, B, nullptr, X, parts, nparts, allow_tc);
+    return launch_dense_energy(ctx, B, nullptr, X, parts, nparts, allow_tc);
 }
 
 }  // namespace vq
