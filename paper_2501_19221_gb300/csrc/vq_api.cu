@@ -148,6 +148,13 @@ int DevBuf::ensure(size_t b) {
     return VELOXQ_OK;
 }
 
+int PinnedWords::make() {
+    VQ_CUDA(cudaHostAlloc(&p, 16, cudaHostAllocMapped));
+    std::memset(p, 0, 16);
+    VQ_CUDA(cudaHostGetDevicePointer(&dev, p, 0));
+    return VELOXQ_OK;
+}
+
 // extra per-context state kept out of the public struct definition
 struct CtxExtra {
     cudaStream_t work = nullptr;
@@ -389,13 +396,14 @@ void tune_store(const std::string& key, int stages, int group) {
 
 // Every call on a context runs on the device the context was created on,
 // which must be the current device: its buffers live there.
-int check_device(const veloxq_ctx* ctx) {
+// A bounded wait that gave up in an earlier asynchronous call is reported here.
+int check_device(veloxq_ctx* ctx) {
     int dev = -1;
     VQ_CUDA(cudaGetDevice(&dev));
     if (dev != ctx->device)
         return fail(VELOXQ_EINVAL, "the context was created on device " + std::to_string(ctx->device) +
                                        ", which must be the current device (current: " + std::to_string(dev) + ")");
-    return VELOXQ_OK;
+    return t32_check(ctx);
 }
 
 int check_err_word(veloxq_ctx* ctx) {
@@ -415,7 +423,7 @@ bool is_readout(const RunParams& p, int k) {
 // (if not null) is recorded right after the last integration step; tc_energy:
 // readout energies in the tensor-core form (sized before the capture).
 int enqueue_loop(veloxq_ctx* ctx, veloxq_path path, int32_t R, const RunParams& p, int nparts, const TcRun* tc,
-                 bool tc_energy, cudaEvent_t ev_steps) {
+                 T32Run* t32, bool tc_energy, cudaEvent_t ev_steps) {
     const Layout lay = path == VELOXQ_PATH_DENSE ? LAYOUT_RN : LAYOUT_NR;
     float* cur = ctx->s_a.as<float>();
     float* nxt = ctx->s_b.as<float>();
@@ -436,12 +444,18 @@ int enqueue_loop(veloxq_ctx* ctx, veloxq_path path, int32_t R, const RunParams& 
                 cb ^= 1;
             }
             k = k1;
+        } else if (t32) {
+            int k1 = k;
+            while (!is_readout(p, k1)) ++k1;
+            VQ_TRY(t32_run(ctx, R, t32, &cur, &nxt, Y, at, k, k1 + 1, p.dt, p.a0, p.c0, nullptr, rule_of(p), false,
+                           false));
+            k = k1;
         } else if (path == VELOXQ_PATH_DENSE) {
             VQ_TRY(dense_step(ctx, R, cur, nxt, Y, at, k, p.dt, p.a0, p.c0, nullptr, rule_of(p)));
         } else {
             VQ_TRY(stream_step(ctx, R, cur, nxt, Y, at, k, p.dt, p.a0, p.c0, nullptr, rule_of(p)));
         }
-        if (!tc) std::swap(cur, nxt);
+        if (!tc && !t32) std::swap(cur, nxt);
         // an event node of the graph (a plain record during capture would only order streams)
         if (ev_steps && k == p.K - 1) VQ_CUDA(cudaEventRecordWithFlags(ev_steps, ctx->stream, cudaEventRecordExternal));
         if (!is_readout(p, k)) continue;
@@ -677,13 +691,21 @@ int veloxq_solve(veloxq_ctx* ctx, int32_t replicas, int32_t steps, const veloxq_
         TcRun tc;
         const bool use_tc = path == VELOXQ_PATH_DENSE && p.prec != VELOXQ_PREC_FP32;
         if (use_tc) VQ_TRY(tc_setup(ctx, p.prec, replicas, &tc, p.method));
-        if (path == VELOXQ_PATH_DENSE && !use_tc) VQ_TRY(dense_prepare(ctx, replicas));
         if (path == VELOXQ_PATH_DENSE) VQ_TRY(tc_energy_prepare(ctx, replicas));
+        // the FP32 field in BF16 terms, unless the start state may leave their range
+        T32Run t32r;
+        bool use_t32 = false;
+        if (path == VELOXQ_PATH_DENSE && !use_tc) {
+            if (p.sigma0 == 0.0f || p.sigma0 >= 6.6174449e-24f /* 2^-77: |s| >= 2^-100 or 0 */)
+                VQ_TRY(t32_prepare(ctx, replicas, &use_t32));
+            if (!use_t32) VQ_TRY(dense_prepare(ctx, replicas));
+        }
         const bool tc_e = path == VELOXQ_PATH_DENSE && tc_energy_ready(ctx, replicas);
         VQ_CUDA(cudaEventRecord(ex->t0, ctx->stream));
         VQ_TRY(launch_init_state(ctx, replicas, seed, p.sigma0, lay, ctx->s_a.as<float>(), ctx->y.as<float>()));
         if (use_tc || tc_e) VQ_CUDA(cudaMemsetAsync(ctx->errw.p, 0, sizeof(int), ctx->stream));
         if (use_tc) VQ_TRY(tc_quant_s(ctx, p.prec, replicas, ctx->s_a.as<float>(), tc.sop[0], rule_of(p)));
+        if (use_t32) VQ_TRY(t32_split(ctx, replicas, ctx->s_a.as<float>(), rule_of(p), false, &t32r));
         VQ_CUDA(cudaMemsetAsync(ctx->best_e.p, 0x7f, sizeof(int64_t) * R, ctx->stream));
         VQ_CUDA(cudaMemsetAsync(ctx->best_bits.p, 0, sizeof(uint32_t) * R * nw, ctx->stream));
         // the captured loop depends on every pointer and parameter below
@@ -697,7 +719,10 @@ int veloxq_solve(veloxq_ctx* ctx, int32_t replicas, int32_t steps, const veloxq_
                                      (uint64_t)(uintptr_t)ctx->xout.p, (uint64_t)(uintptr_t)ctx->a_table.p};
         key.push_back((uint64_t)p.method);
         for (uint64_t v : {(uint64_t)tc_e, (uint64_t)ctx->eplanes, (uint64_t)(uintptr_t)ctx->eplane.p,
-                           (uint64_t)(uintptr_t)ctx->exop.p, (uint64_t)(uintptr_t)ctx->efield.p})
+                           (uint64_t)(uintptr_t)ctx->exop.p, (uint64_t)(uintptr_t)ctx->efield.p,
+                           (uint64_t)use_t32, (uint64_t)(uintptr_t)ctx->q3.p, (uint64_t)(uintptr_t)ctx->s3[0].p,
+                           (uint64_t)(uintptr_t)ctx->s3[1].p, (uint64_t)(uintptr_t)ctx->dpart.p,
+                           (uint64_t)(uintptr_t)ctx->tcdone.p})
             key.push_back(v);
         float fp[4] = {p.dt, p.a0, p.c0, p.alpha};
         for (float f : fp) {
@@ -712,7 +737,8 @@ int veloxq_solve(veloxq_ctx* ctx, int32_t replicas, int32_t steps, const veloxq_
             }
             cudaGraph_t g = nullptr;
             VQ_CUDA(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
-            int st = enqueue_loop(ctx, path, replicas, p, nparts, use_tc ? &tc : nullptr, tc_e, ex->t2);
+            int st = enqueue_loop(ctx, path, replicas, p, nparts, use_tc ? &tc : nullptr,
+                                  use_t32 ? &t32r : nullptr, tc_e, ex->t2);
             cudaError_t ce = cudaStreamEndCapture(ctx->stream, &g);
             if (st != VELOXQ_OK) {
                 if (g) cudaGraphDestroy(g);
@@ -733,8 +759,16 @@ int veloxq_solve(veloxq_ctx* ctx, int32_t replicas, int32_t steps, const veloxq_
         VQ_CUDA(cudaEventRecord(ex->t1, ctx->stream));
         VQ_CUDA(cudaGraphLaunch(ex->graph, ctx->stream));   // records t2 after the last step
         VQ_CUDA(cudaEventRecord(ex->t3, ctx->stream));
-        launches = 1 + (use_tc ? 1 : 0) + ex->graph_launches;   // init (+ operand) kernels + graph nodes
+        launches = 1 + (use_tc || use_t32 ? 1 : 0) + ex->graph_launches;   // init (+ operand) kernels + graph nodes
         main_launches = steps;
+        if (use_t32) {
+            main_launches = 0;
+            for (int k = 0, from = 0; k < steps; ++k)
+                if (is_readout(p, k)) {
+                    main_launches += t32_launches(ctx, replicas, k + 1 - from);
+                    from = k + 1;
+                }
+        }
         if (use_tc) {
             // one launch per run of steps up to a readout
             main_launches = 0;
@@ -749,6 +783,7 @@ int veloxq_solve(veloxq_ctx* ctx, int32_t replicas, int32_t steps, const veloxq_
     if (x_best) VQ_CUDA(cudaMemcpyAsync(x_best, ctx->xout.p, (size_t)n, cudaMemcpyDeviceToHost, ctx->stream));
     VQ_CUDA(cudaStreamSynchronize(ctx->stream));
     VQ_LAUNCH_CHECK("solve");
+    VQ_TRY(t32_check(ctx));
     {
         float a = 0.f, b = 0.f;
         VQ_CUDA(cudaEventElapsedTime(&a, ex->t0, ex->t3));
@@ -971,7 +1006,17 @@ int veloxq_field_dev(veloxq_ctx* ctx, int32_t R, veloxq_prec prec, const float* 
     if (R < 1 || R > kMaxReplicas || !S || !F) return fail(VELOXQ_EINVAL, "R in [1, 2^20] and non-NULL S, F required");
     if (prec < VELOXQ_PREC_FP32 || prec > VELOXQ_PREC_FP8_ONE_TERM) return fail(VELOXQ_EINVAL, "unknown precision");
     if (ctx->dense) {
-        if (prec == VELOXQ_PREC_FP32) return dense_field(ctx, R, S, F);
+        if (prec == VELOXQ_PREC_FP32) {
+            bool t32 = false;
+            VQ_TRY(t32_prepare(ctx, R, &t32));
+            if (!t32) return dense_field(ctx, R, S, F);
+            // S may hold anything: where a value leaves the terms' range the tensor-core kernels do nothing
+            // and the SGEMM runs, else the other way round
+            T32Run t;
+            VQ_TRY(t32_split(ctx, R, S, Rule(), true, &t));
+            VQ_TRY(t32_run(ctx, R, &t, nullptr, nullptr, nullptr, nullptr, 0, 1, 0.f, 0.f, 0.f, F, Rule(), true, true));
+            return dense_field(ctx, R, S, F, ctx->t32w.as<uint32_t>() + 1, t.seq);
+        }
         TcRun tc;
         VQ_TRY(tc_setup(ctx, prec, R, &tc));
         VQ_CUDA(cudaMemsetAsync(ctx->errw.p, 0, sizeof(int), ctx->stream));
@@ -1000,18 +1045,33 @@ int veloxq_steps_dev(veloxq_ctx* ctx, int32_t R, int32_t k_begin, int32_t k_coun
     VQ_TRY(resolve(ctx, sched, K, &p));
     const veloxq_path path = choose_path(ctx, p.path, p.prec, R);
     VQ_TRY(check_path(ctx, path, p.prec, R));
-    VQ_TRY(upload_schedule(ctx, p));
     const int64_t n = ctx->n, nR = n * (int64_t)R;
     const int k_end = k_begin + k_count;
+    T32Run t32r;
+    bool t32 = false;
+    if (path == VELOXQ_PATH_DENSE && p.prec == VELOXQ_PREC_FP32) {
+        VQ_TRY(t32_prepare(ctx, R, &t32));
+        if (t32) VQ_TRY(t32_split(ctx, R, S, rule_of(p), true, &t32r));
+    }
+    VQ_TRY(upload_schedule(ctx, p));   // waits for the stream, so for the range check of the split too
+    if (t32 && t32_bad(ctx, t32r)) t32 = false;
     if (path == VELOXQ_PATH_RESIDENT)
         return resident_run(ctx, R, p, 0, k_begin, k_end, S, Y, S, Y, F_last, nullptr, nullptr);
-    VQ_TRY(ctx->s_a.ensure(sizeof(float) * nR));
     VQ_TRY(ctx->s_b.ensure(sizeof(float) * nR));
     const float* at = ctx->a_table.as<float>();
-    float* cur = ctx->s_a.as<float>();
     float* nxt = ctx->s_b.as<float>();
     if (path == VELOXQ_PATH_DENSE) {
-        VQ_CUDA(cudaMemcpyAsync(cur, S, sizeof(float) * nR, cudaMemcpyDeviceToDevice, ctx->stream));
+        // the caller's S is one of the two state buffers: no copy unless the state ends in the other
+        float* cur = S;
+        auto give_back = [&]() -> int {
+            if (cur != S) VQ_CUDA(cudaMemcpyAsync(S, cur, sizeof(float) * nR, cudaMemcpyDeviceToDevice, ctx->stream));
+            return VELOXQ_OK;
+        };
+        if (t32) {
+            VQ_TRY(t32_run(ctx, R, &t32r, &cur, &nxt, Y, at, k_begin, k_end, p.dt, p.a0, p.c0, F_last, rule_of(p), false,
+                           false));
+            return give_back();
+        }
         if (p.prec != VELOXQ_PREC_FP32) {
             TcRun tc;
             VQ_TRY(tc_setup(ctx, p.prec, R, &tc, p.method));
@@ -1021,7 +1081,7 @@ int veloxq_steps_dev(veloxq_ctx* ctx, int32_t R, int32_t k_begin, int32_t k_coun
             VQ_TRY(tc_run(ctx, p.prec, R, tc.mq, tc.ms, tc.lo(), 0, cur, nxt, Y, tc.sop, at, k_begin, k_end, p.dt,
                           p.a0, p.c0, F_last, ctx->errw.as<int>(), rule_of(p)));
             if (k_count & 1) std::swap(cur, nxt);
-            VQ_CUDA(cudaMemcpyAsync(S, cur, sizeof(float) * nR, cudaMemcpyDeviceToDevice, ctx->stream));
+            VQ_TRY(give_back());
             return check_err_word(ctx);
         }
         for (int k = k_begin; k < k_end; ++k) {
@@ -1029,9 +1089,10 @@ int veloxq_steps_dev(veloxq_ctx* ctx, int32_t R, int32_t k_begin, int32_t k_coun
                               rule_of(p)));
             std::swap(cur, nxt);
         }
-        VQ_CUDA(cudaMemcpyAsync(S, cur, sizeof(float) * nR, cudaMemcpyDeviceToDevice, ctx->stream));
-        return VELOXQ_OK;
+        return give_back();
     }
+    VQ_TRY(ctx->s_a.ensure(sizeof(float) * nR));
+    float* cur = ctx->s_a.as<float>();
     VQ_TRY(ctx->y.ensure(sizeof(float) * nR));
     VQ_TRY(ctx->f.ensure(sizeof(float) * nR));
     VQ_TRY(launch_transpose(ctx->stream, S, cur, R, n));

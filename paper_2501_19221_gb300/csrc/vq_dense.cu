@@ -41,7 +41,9 @@ __global__ void __launch_bounds__(256) k_dense_step(int32_t R, int32_t n, const 
                                                     float* __restrict__ Y, const float* __restrict__ bf,
                                                     const float* __restrict__ a_table, int k, float dt, float a0,
                                                     float c0, float* __restrict__ F_out, int method, float alpha,
-                                                    int ktile_per, float* __restrict__ part) {
+                                                    int ktile_per, float* __restrict__ part,
+                                                    const uint32_t* only, uint32_t only_seq) {
+    if (only && *only != only_seq) return;
     __shared__ __align__(16) float As[2][BK][BM];
     __shared__ __align__(16) float Bs[ASYNC ? BST : 2][BK][BN];
     const int tid = threadIdx.x;
@@ -198,7 +200,9 @@ __global__ void __launch_bounds__(256) k_dense_finish(int32_t R, int32_t n, int 
                                                       const float* __restrict__ S_cur, float* __restrict__ S_nxt,
                                                       float* __restrict__ Y, const float* __restrict__ bf,
                                                       const float* __restrict__ a_table, int k, float dt, float a0,
-                                                      float c0, float* __restrict__ F_out, int method, float alpha) {
+                                                      float c0, float* __restrict__ F_out, int method, float alpha,
+                                                      const uint32_t* only, uint32_t only_seq) {
+    if (only && *only != only_seq) return;
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t total = (int64_t)R * n;
     if (p >= total) return;
@@ -243,7 +247,8 @@ void dense_split(int64_t n, int32_t R, int sms, int* ksplit, int* per) {
 
 template <bool FIELD_ONLY>
 int launch_dense_step(veloxq_ctx* ctx, int32_t R, const float* S_cur, float* S_nxt, float* Y, const float* a_table,
-                      int k, float dt, float a0, float c0, float* F_out, const Rule& rule) {
+                      int k, float dt, float a0, float c0, float* F_out, const Rule& rule,
+                      const uint32_t* only = nullptr, uint32_t only_seq = 0) {
     const int32_t n = (int32_t)ctx->n;
     int ksplit, per;
     dense_split(n, R, device_sms(ctx->device), &ksplit, &per);
@@ -266,15 +271,17 @@ int launch_dense_step(veloxq_ctx* ctx, int32_t R, const float* S_cur, float* S_n
     if (async_b)
         k_dense_step<FIELD_ONLY, true><<<g, 256, 0, ctx->stream>>>(R, n, S_cur, ctx->qoff32.as<float>(), S_nxt, Y,
                                                                    ctx->bf.as<float>(), a_table, k, dt, a0, c0,
-                                                                   F_out, rule.method, rule.alpha, per, part);
+                                                                   F_out, rule.method, rule.alpha, per, part, only,
+                                                                   only_seq);
     else
         k_dense_step<FIELD_ONLY, false><<<g, 256, 0, ctx->stream>>>(R, n, S_cur, ctx->qoff32.as<float>(), S_nxt, Y,
                                                                     ctx->bf.as<float>(), a_table, k, dt, a0, c0,
-                                                                    F_out, rule.method, rule.alpha, per, part);
+                                                                    F_out, rule.method, rule.alpha, per, part, only,
+                                                                   only_seq);
     if (ksplit > 1)
         k_dense_finish<FIELD_ONLY><<<(unsigned)div_up((int64_t)R * n, 256), 256, 0, ctx->stream>>>(
             R, n, ksplit, part, S_cur, S_nxt, Y, ctx->bf.as<float>(), a_table, k, dt, a0, c0, F_out, rule.method,
-            rule.alpha);
+            rule.alpha, only, only_seq);
     VQ_LAUNCH_CHECK("dense_step");
     return VELOXQ_OK;
 }
@@ -326,8 +333,8 @@ int dense_prepare(veloxq_ctx* ctx, int32_t R) {
     return VELOXQ_OK;
 }
 
-int dense_field(veloxq_ctx* ctx, int32_t R, const float* S, float* F) {
-    return launch_dense_step<true>(ctx, R, S, nullptr, nullptr, nullptr, 0, 0.f, 0.f, 0.f, F, Rule());
+int dense_field(veloxq_ctx* ctx, int32_t R, const float* S, float* F, const uint32_t* only, uint32_t only_seq) {
+    return launch_dense_step<true>(ctx, R, S, nullptr, nullptr, nullptr, 0, 0.f, 0.f, 0.f, F, Rule(), only, only_seq);
 }
 
 // allow_tc: the tensor-core form when tc_energy_prepare has sized it for R

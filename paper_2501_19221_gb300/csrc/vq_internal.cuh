@@ -56,6 +56,20 @@ struct DevBuf {
     template <typename T> T* as() const { return static_cast<T*>(p); }
 };
 
+// Four zeroed words of mapped host memory that kernels write in rare cases
+// and the host reads without a copy.
+struct PinnedWords {
+    void* p = nullptr;
+    void* dev = nullptr;        // device address
+    PinnedWords() = default;
+    PinnedWords(const PinnedWords&) = delete;
+    PinnedWords& operator=(const PinnedWords&) = delete;
+    ~PinnedWords() {
+        if (p) cudaFreeHost(p);
+    }
+    int make();
+};
+
 // Row layout of a state block in device memory.
 enum Layout { LAYOUT_RN = 0 /* [R][n], replica-major */, LAYOUT_NR = 1 /* [n][R] */ };
 
@@ -127,6 +141,13 @@ struct veloxq_ctx {
     vq::DevBuf s_a, s_b, y, f, ework, best_e, best_bits, flags, a_table, xout, misc;
     vq::DevBuf sop_a, sop_b;      // tensor-core operand copies of S (ping-pong)
     vq::DevBuf dpart;             // float [ksplit][R][n] split-k partial fields of the FP32 dense step
+    // FP32 field on the tensor cores (vq_tc32.cu)
+    int q3_state = 0;             // term planes of Qoff: 0 not built yet, 1 built, -1 not used
+    vq::DevBuf q3;                // bf16 [3][n][n_pad] Qoff in three exact terms
+    vq::DevBuf s3[2];             // bf16 [3][R][n_pad] operand terms of S (ping-pong)
+    vq::DevBuf t32w;              // [0] error word of its waits, [1] sequence number of the last operand out of range
+    vq::PinnedWords t32h;         // the same two words where the host can see them without a copy
+    uint32_t t32_seq = 0;
     vq::DevBuf errw;              // device error word of bounded waits
     vq::DevBuf tcdone;            // uint32 [replica column blocks] completion counters of a tensor-core run
     int stream_unroll = 0;        // gather variant of the streaming kernels: 1, 4, or 6 (rows of exactly
@@ -187,7 +208,9 @@ int resident_run(veloxq_ctx* ctx, int32_t R, const RunParams& p, uint64_t seed, 
 // dense kernels (vq_dense.cu)
 int dense_step(veloxq_ctx* ctx, int32_t R, const float* S_cur, float* S_nxt, float* Y,
                const float* a_table, int k, float dt, float a0, float c0, float* F_out, const Rule& rule = Rule());
-int dense_field(veloxq_ctx* ctx, int32_t R, const float* S, float* F);
+// only (or null): the kernels do nothing unless *only == only_seq
+int dense_field(veloxq_ctx* ctx, int32_t R, const float* S, float* F, const uint32_t* only = nullptr,
+                uint32_t only_seq = 0);
 int dense_prepare(veloxq_ctx* ctx, int32_t R);   // workspace of the split-k FP32 step (before capture)
 int dense_energy(veloxq_ctx* ctx, int32_t R, const float* S, int64_t* parts, int* nparts, bool allow_tc);
 int dense_energy_x(veloxq_ctx* ctx, int64_t B, const uint8_t* X, int64_t* parts, int* nparts, bool allow_tc);
@@ -249,6 +272,21 @@ int tc_field(veloxq_ctx* ctx, int prec, int32_t R, const CUtensorMap& mq, const 
              const CUtensorMap* ms_lo, float* F_out, int* err);
 int tc_operand_map(CUtensorMap* m, void* base, int prec, int64_t rows, int64_t n_pad, bool a_operand);
 int launch_sum_parts(veloxq_ctx* ctx, int64_t B, int nparts, const int64_t* parts, double* E, int64_t* E_int);
+
+// FP32 field on the tensor cores (vq_tc32.cu): the operand state of a run.
+struct T32Run {
+    int cur = 0;          // operand buffer of the next step
+    int terms = 3;        // BF16 terms of the operand
+    uint32_t seq = 0;     // sequence number of its range check (0: not checked)
+};
+int t32_prepare(veloxq_ctx* ctx, int32_t R, bool* ready);
+int t32_split(veloxq_ctx* ctx, int32_t R, const float* S, const Rule& rule, bool check, T32Run* t);
+bool t32_bad(const veloxq_ctx* ctx, const T32Run& t);
+int t32_launches(const veloxq_ctx* ctx, int32_t R, int steps);
+int t32_run(veloxq_ctx* ctx, int32_t R, T32Run* t, float** cur, float** nxt, float* Y, const float* a_table,
+            int k_begin, int k_end, float dt, float a0, float c0, float* F_out, const Rule& rule, bool field_only,
+            bool guard);
+int t32_check(veloxq_ctx* ctx);
 
 // exact readout energies of a dense instance on the tensor cores (vq_energy_tc.cu)
 int tc_energy_prepare(veloxq_ctx* ctx, int64_t R);   // digit planes and workspaces (before capture)

@@ -41,10 +41,13 @@
 #include <cstdlib>
 
 #include "vq_internal.cuh"
+#include "vq_tc.cuh"
 
 namespace vq {
 
 namespace {
+
+using namespace tc;
 
 // BM rows per CTA (2 BM per pair), BN replicas per pair (BN / 2 staged per CTA)
 constexpr int BM = 128, BN = 256, BNH = BN / 2, BKB = 128;
@@ -55,149 +58,6 @@ template <int TERMS> constexpr int stages_of() { return TERMS == 2 ? 4 : 6; }
 constexpr uint32_t PIPE_BYTES = 6 * stage_bytes<1>();
 static_assert(stages_of<2>() * stage_bytes<2>() == PIPE_BYTES, "both stage forms fill the same 192 KB");
 constexpr size_t TC_SMEM = (size_t)PIPE_BYTES + 1024 /*align*/ + 256 /*barriers, tensor-memory slot*/;
-constexpr long long kWaitCycles = 4000000000LL;   // ~2 s at 2 GHz
-
-enum { TC_ERR_PRODUCER = 1, TC_ERR_MMA = 2, TC_ERR_EPILOGUE = 4, TC_ERR_SELFTEST = 8, TC_ERR_DEPEND = 16 };
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-// The same with cluster-scope acquire, for barriers the peer CTA arrives on.
-__device__ __forceinline__ bool mbar_try_wait_cl(uint64_t* bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-// Bounded wait: false (and the error word set) if the phase does not complete
-// within the budget or another thread already gave up.
-template <bool CLUSTER = false>
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* err, int code,
-                                          long long budget = kWaitCycles) {
-    const long long t0 = clock64();
-    uint32_t spins = 0;
-    while (!(CLUSTER ? mbar_try_wait_cl(bar, parity) : mbar_try_wait(bar, parity))) {
-        if ((++spins & 1023u) == 0) {
-            if (*(volatile int*)err) return false;
-            if (clock64() - t0 > budget) {
-                atomicOr(err, code);
-                return false;
-            }
-        }
-    }
-    return true;
-}
-
-// ---- cluster of two CTAs ----
-__device__ __forceinline__ uint32_t cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-// shared::cluster address of the same shared variable in CTA `rank`
-__device__ __forceinline__ uint32_t mapa(uint32_t a, uint32_t rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-    return r;
-}
-__device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void mbar_arrive_remote(uint32_t cl_addr) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cl_addr) : "memory");
-}
-
-// 2-D tile load into this CTA's shared memory; completion is counted on the
-// barrier at cluster address `bar_cl` (the even CTA's barrier of the pair).
-__device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* map, int x, int y, uint32_t bar_cl) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 "
-        "[%0], [%1, {%2, %3}], [%4];"
-        ::"r"(smem_u32(dst)), "l"((uint64_t)map), "r"(x), "r"(y), "r"(bar_cl)
-        : "memory");
-}
-// The same with an L2 cache policy (the coupling operand, which every column
-// block of every step reads again, is kept in L2 ahead of streaming data).
-__device__ __forceinline__ void tma_load_2d_pair_hint(void* dst, const CUtensorMap* map, int x, int y,
-                                                      uint32_t bar_cl, uint64_t pol) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2.L2::cache_hint "
-        "[%0], [%1, {%2, %3}], [%4], %5;"
-        ::"r"(smem_u32(dst)), "l"((uint64_t)map), "r"(x), "r"(y), "r"(bar_cl), "l"(pol)
-        : "memory");
-}
-__device__ __forceinline__ uint64_t l2_evict_last_policy() {
-    uint64_t pol;
-    asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
-    return pol;
-}
-
-// ---- completion counters between CTAs of one grid (steps of a run) ----
-__device__ __forceinline__ uint32_t ld_acquire_u32(const uint32_t* p) {
-    uint32_t v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ void red_release_add(uint32_t* p, uint32_t v) {
-    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-// Generic-proxy writes to global memory made visible to (and ordered with)
-// the async proxy: the bulk tensor copies of another CTA read them.
-__device__ __forceinline__ void fence_proxy_async_global() {
-    asm volatile("fence.proxy.async.global;" ::: "memory");
-}
-// Bounded wait until *c >= target: false (and the error word set) if it is
-// not reached within the budget or another thread already gave up.
-__device__ __forceinline__ bool count_wait(const uint32_t* c, uint32_t target, int* err, int code) {
-    const long long t0 = clock64();
-    uint32_t spins = 0;
-    while (ld_acquire_u32(c) < target) {
-        if ((++spins & 255u) == 0) {
-            if (*(volatile int*)err) return false;
-            if (clock64() - t0 > kWaitCycles) {
-                atomicOr(err, code);
-                return false;
-            }
-        }
-    }
-    return true;
-}
-
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-// Tensor memory of a CTA pair: one warp of each CTA allocates (and frees)
-// together; both CTAs receive the same column address.
-__device__ __forceinline__ void tmem_alloc(uint32_t* slot, uint32_t ncols) {
-    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)), "r"(ncols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
-    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
-}
-
 // Shared-memory matrix descriptor: K-major operand, 128-byte swizzle, 8-row
 // core groups 1024 bytes apart.
 __device__ __forceinline__ uint64_t smem_desc(const void* p) {
@@ -240,26 +100,6 @@ __device__ __forceinline__ void umma(uint32_t d_tmem, uint64_t a, uint64_t b, ui
             : "memory");
     }
 }
-// Arrive on the barrier at the same offset in both CTAs once the MMAs issued
-// so far have completed.
-__device__ __forceinline__ void umma_commit_pair(uint64_t* bar) {
-    asm volatile(
-        "{\n\t.reg .b16 m;\n\tmov.b16 m, 3;\n\t"
-        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], m;\n\t}\n"
-        ::"r"(smem_u32(bar))
-        : "memory");
-}
-
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
 struct TcArgs {
     int32_t n, R, n_pad;
     int32_t k, k_end;        // steps k .. k_end - 1 of the schedule (one launch)
