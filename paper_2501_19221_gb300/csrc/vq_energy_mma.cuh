@@ -4,7 +4,7 @@
 // k_batch_energy).
 //
 // The fixed-point couplings q_ij = round(Q_ij 2^S) are written in balanced
-// base-4096 digits, q = sum_k 4096^k t_k with t_k in [-2048, 2047], which FP16
+// base-4096 digits, q = sum_k 4096^k t_k with t_k in [-2048, 2048], which FP16
 // holds exactly. A block stages 64 rows x 64 columns of Q at a time, extracts
 // one digit plane after the other into shared memory (only as many as the
 // tile's largest |q| needs: one for small integers, four for Gaussian FP32
@@ -215,58 +215,74 @@ __device__ __forceinline__ void energy_tile(Smem<TR>& sm, int64_t R, int32_t n, 
         }
     };
 
-    // with C = sum_{k < 5} 2048 4096^k added, digit k < 5 of q is the k-th
-    // 12-bit field less 2048, and digit 5 what is left above
+    // The couplings of a stage as their fixed-point values: FP32 and int8
+    // couplings times 2^shift are exact in FP32, and their digits come from
+    // the top down by rounding (the last one is the rounding to an integer,
+    // ties to even). The other types take int64 values with
+    // C = sum_{k < 5} 2048 4096^k added, so that digit k < 5 is the k-th
+    // 12-bit field less 2048 and digit 5 what is left above.
+    constexpr bool kFloat = std::is_same<QT, float>::value || std::is_same<QT, int8_t>::value;
+    using Val = std::conditional_t<kFloat, float, long long>;
     constexpr long long kOffset = 2048ll * (1ll + (1ll << 12) + (1ll << 24) + (1ll << 36) + (1ll << 48));
+    const float f1 = ldexpf(1.0f, min(shift, 100)), f2 = ldexpf(1.0f, max(0, shift - 100));
     float low[4][4];                                   // the lowest digit's sums, over up to FLUSH stages
     zero(low);
     int buf = 0, stage = 0, since = 0;
     for (int32_t j0 = 0; j0 < n; j0 += TK, ++stage) {
-        long long q[EQ][2];
+        Val q[EQ][2];
         uint32_t m = 0;
 #pragma unroll
         for (int e = 0; e < EQ; ++e)
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                q[e][h] = vqd::qfix<QT>(raw[e].v[h], shift) + kOffset;
+                if constexpr (kFloat) q[e][h] = (float)raw[e].v[h] * f1 * f2;
+                else q[e][h] = vqd::qfix<QT>(raw[e].v[h], shift) + kOffset;
                 m = max(m, mag(raw[e].v[h]));
             }
         m = __reduce_max_sync(0xffffffffu, m);
         // L digits hold every |q| < 2^(12 L - 2)
         if (lane == 0) sm.digits[stage & 1][warp] = (uint32_t)max(1, min(6, (bits_of<QT>(m, shift) + 13) / 12));
-        auto store_digit = [&](int k) {
+        __syncthreads();                               // digit counts; the previous stage's products have read sm.b
+        uint32_t digits = 1;
 #pragma unroll
-            for (int e = 0; e < EQ; ++e) {
-                float f[2];
-#pragma unroll
-                for (int h = 0; h < 2; ++h)
-                    f[h] = k < 5 ? __uint_as_float(((uint32_t)((unsigned long long)q[e][h] >> (12 * k)) & 4095u) |
-                                                   0x4B000000u) - 8390656.0f           // 2^23 + 2048
-                                 : (float)(int)(q[e][h] >> 60);
-                *reinterpret_cast<__half2*>(&sm.a[buf][warp + WARPS * e][2 * lane]) = __floats2half2_rn(f[0], f[1]);
-            }
-        };
-        if (stage) __syncthreads();                    // the previous stage's products have read sm.b and its planes
-        store_digit(0);
+        for (int w = 0; w < WARPS / 4; ++w) {
+            const uint4 d = reinterpret_cast<const uint4*>(sm.digits[stage & 1])[w];
+            digits = max(digits, max(max(d.x, d.y), max(d.z, d.w)));
+        }
 #pragma unroll
         for (int e = 0; e < EX; ++e)
             *reinterpret_cast<uint32_t*>(&sm.b[warp + WARPS * e][2 * lane]) =
                 (is_on(xr[e].v[0]) ? 0x3C00u : 0u) | (is_on(xr[e].v[1]) ? 0x3C000000u : 0u);
         if (j0 + TK < n) load(j0 + TK);
-        __syncthreads();
-        product(buf, low);
-        buf ^= 1;
-        uint32_t digits = 1;
+        // The plane before last is overwritten: every warp read it before the barrier that published the last one
+        for (int k = (int)digits - 1; k >= 0; --k) {
+            const float down = __int_as_float((127 - 12 * k) << 23), up = __int_as_float((127 + 12 * k) << 23);
 #pragma unroll
-        for (int w = 0; w < WARPS; ++w) digits = max(digits, sm.digits[stage & 1][w]);
-        for (int k = 1; k < (int)digits; ++k) {
-            store_digit(k);                            // the plane before last: read by every warp before the
-            __syncthreads();                           // barrier that published the last one
-            float acc[4][4];
-            zero(acc);
-            product(buf, acc);
+            for (int e = 0; e < EQ; ++e) {
+                float f[2];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    if constexpr (kFloat) {
+                        f[h] = __fsub_rn(fmaf(q[e][h], down, 12582912.0f), 12582912.0f);   // rounded: |.| <= 2048
+                        q[e][h] = fmaf(-f[h], up, q[e][h]);                                // exact
+                    } else {
+                        f[h] = k < 5 ? __uint_as_float(((uint32_t)((unsigned long long)q[e][h] >> (12 * k)) & 4095u) |
+                                                       0x4B000000u) - 8390656.0f           // 2^23 + 2048
+                                     : (float)(int)(q[e][h] >> 60);
+                    }
+                }
+                *reinterpret_cast<__half2*>(&sm.a[buf][warp + WARPS * e][2 * lane]) = __floats2half2_rn(f[0], f[1]);
+            }
+            __syncthreads();
+            if (k == 0) {
+                product(buf, low);
+            } else {
+                float acc[4][4];
+                zero(acc);
+                product(buf, acc);
+                add(acc, 12 * k);
+            }
             buf ^= 1;
-            add(acc, 12 * k);
         }
         if (++since == FLUSH) {
             add(low, 0);
