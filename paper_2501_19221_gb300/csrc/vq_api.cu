@@ -306,7 +306,7 @@ int tc_setup(veloxq_ctx* ctx, int prec, int32_t R, TcRun* t, int method = VELOXQ
     VQ_TRY(ctx->sop_b.ensure(b));
     VQ_TRY(ctx->errw.ensure(sizeof(int) * 4));
     // completion counters of multi-step runs, one per replica column block (sized before any capture)
-    VQ_TRY(ctx->tcdone.ensure(sizeof(uint32_t) * (size_t)div_up(R, 256)));
+    VQ_TRY(ctx->tcdone.ensure(sizeof(uint32_t) * (size_t)div_up(R, 64)));
     // the K padding columns [n, n_pad) of both operand buffers must stay zero:
     // the epilogue never writes them
     VQ_CUDA(cudaMemsetAsync(ctx->sop_a.p, 0, b, ctx->stream));

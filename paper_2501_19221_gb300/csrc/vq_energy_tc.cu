@@ -195,11 +195,11 @@ int tc_energy(veloxq_ctx* ctx, int64_t R, const float* S, const uint8_t* X, int6
     else k_xop<false><<<(unsigned)div_up(total, 256), 256, 0, st>>>(R, n, np, S, nullptr, xop);
     VQ_LAUNCH_CHECK("energy operand");
     CUtensorMap mx;
-    VQ_TRY(tc_operand_map(&mx, xop, VELOXQ_PREC_BF16, R, np, false));
+    VQ_TRY(tc_operand_map(ctx, &mx, xop, VELOXQ_PREC_BF16, R, np, false));
     const dim3 cg((unsigned)div_up(n, 64), (unsigned)std::min<int64_t>(div_up(R, 4), 65535));
     for (int k = 0; k < ctx->eplanes; ++k) {
         CUtensorMap mp;
-        VQ_TRY(tc_operand_map(&mp, ctx->eplane.as<__nv_bfloat16>() + (size_t)k * n * np, VELOXQ_PREC_BF16, n, np, true));
+        VQ_TRY(tc_operand_map(ctx, &mp, ctx->eplane.as<__nv_bfloat16>() + (size_t)k * n * np, VELOXQ_PREC_BF16, n, np, true));
         VQ_TRY(tc_field(ctx, VELOXQ_PREC_BF16, (int32_t)R, mp, mx, nullptr, ctx->efield.as<float>(),
                         ctx->errw.as<int>()));
         if (X)

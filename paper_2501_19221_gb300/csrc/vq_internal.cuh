@@ -270,7 +270,8 @@ int tc_run(veloxq_ctx* ctx, int prec, int32_t R, const CUtensorMap& mq, const CU
 // The field alone, F = Qoff S, of the operand behind ms (and ms_lo).
 int tc_field(veloxq_ctx* ctx, int prec, int32_t R, const CUtensorMap& mq, const CUtensorMap& ms,
              const CUtensorMap* ms_lo, float* F_out, int* err);
-int tc_operand_map(CUtensorMap* m, void* base, int prec, int64_t rows, int64_t n_pad, bool a_operand);
+int tc_tile(const veloxq_ctx* ctx, int prec, int terms, int32_t R);   // replicas per tile: 256, 128 or 64
+int tc_operand_map(veloxq_ctx* ctx, CUtensorMap* m, void* base, int prec, int64_t rows, int64_t n_pad, bool a_operand);
 int launch_sum_parts(veloxq_ctx* ctx, int64_t B, int nparts, const int64_t* parts, double* E, int64_t* E_int);
 
 // FP32 field on the tensor cores (vq_tc32.cu): the operand state of a run.

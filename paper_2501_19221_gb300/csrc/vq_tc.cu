@@ -6,8 +6,9 @@
 // replicas, K = variables. Both operands are K-major (Qoff row-major, S
 // replica-major), 128-byte K blocks with the 128-byte swizzle.
 // CTA pairs (clusters of 2, tcgen05 cta_group::2): a pair computes a
-// 256 x 256 tile with M = 256 MMAs issued by the even CTA. Each CTA stages
-// its own 128 rows of Qoff and its own 128 replicas of S; each CTA's tensor
+// 256 x 256 tile (256 x 128 or 256 x 64 where wide tiles would leave pairs
+// idle, tc_tile) with M = 256 MMAs issued by the even CTA. Each CTA stages
+// its own 128 rows of Qoff and its own half of the tile's replicas of S; each CTA's tensor
 // memory holds the accumulator of its 128 rows for all 256 replicas.
 //   BF16: Qop = bf16(Qoff), Sop = bf16(s)                (kind::f16)
 //   FP8 : Qop = e4m3(Qoff_ij / q_i), q_i = amax_i / 448  (kind::f8f6f4)
@@ -38,6 +39,7 @@
 #include <cuda_fp8.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstdlib>
 
 #include "vq_internal.cuh"
@@ -49,14 +51,17 @@ namespace {
 
 using namespace tc;
 
-// BM rows per CTA (2 BM per pair), BN replicas per pair (BN / 2 staged per CTA)
-constexpr int BM = 128, BN = 256, BNH = BN / 2, BKB = 128;
-constexpr uint32_t A_BYTES = BM * BKB, B_BYTES = BNH * BKB;
+// BM rows per CTA (2 BM per pair), BN replicas per pair (a template parameter
+// of the kernel: 256, 128 or 64; BN / 2 staged per CTA)
+constexpr int BM = 128, BKB = 128;
+constexpr int kMaxDevices = 64;
+constexpr uint32_t A_BYTES = BM * BKB;
+template <int BN> constexpr uint32_t b_bytes() { return (BN / 2) * BKB; }
 // a stage holds the Qop block and TERMS blocks of Sop
-template <int TERMS> constexpr uint32_t stage_bytes() { return A_BYTES + TERMS * B_BYTES; }
-template <int TERMS> constexpr int stages_of() { return TERMS == 2 ? 4 : 6; }
-constexpr uint32_t PIPE_BYTES = 6 * stage_bytes<1>();
-static_assert(stages_of<2>() * stage_bytes<2>() == PIPE_BYTES, "both stage forms fill the same 192 KB");
+template <int TERMS, int BN> constexpr uint32_t stage_bytes() { return A_BYTES + TERMS * b_bytes<BN>(); }
+constexpr uint32_t PIPE_BYTES = 6 * stage_bytes<1, 256>();
+template <int TERMS, int BN> constexpr int stages_of() { return (int)(PIPE_BYTES / stage_bytes<TERMS, BN>()); }
+static_assert(stages_of<2, 256>() * stage_bytes<2, 256>() == PIPE_BYTES, "both stage forms fill the same 192 KB");
 constexpr size_t TC_SMEM = (size_t)PIPE_BYTES + 1024 /*align*/ + 256 /*barriers, tensor-memory slot*/;
 // Shared-memory matrix descriptor: K-major operand, 128-byte swizzle, 8-row
 // core groups 1024 bytes apart.
@@ -73,7 +78,7 @@ __device__ __forceinline__ uint64_t smem_desc(const void* p) {
 
 // Instruction descriptor: FP32 accumulator, A/B format, K-major, N, M (the
 // pair's M = 2 BM).
-template <int PREC> __host__ __device__ constexpr uint32_t instr_desc() {
+template <int PREC, int BN> __host__ __device__ constexpr uint32_t instr_desc() {
     return (1u << 4)                                   // D format F32
            | ((PREC == 1 ? 1u : 0u) << 7)              // A: BF16 (f16 kind) / E4M3 (f8f6f4 kind)
            | ((PREC == 1 ? 1u : 0u) << 10)             // B: same
@@ -164,14 +169,16 @@ __device__ __forceinline__ void store_op(void* base, int64_t idx, int64_t plane,
 // METHOD: the integrator (veloxq_method), a template parameter so that each
 // form keeps its own register allocation. TERMS: S operand terms (1, or 2 for
 // FP8 hi + lo; tmL* map the lo planes, unused with one term).
-template <int PREC, int TERMS, bool FIELD_ONLY, int METHOD>
+template <int PREC, int TERMS, int BN, bool FIELD_ONLY, int METHOD>
 __global__ void __launch_bounds__(320, 1) k_tc_step(const __grid_constant__ CUtensorMap tmA,
                                                     const __grid_constant__ CUtensorMap tmB0,
                                                     const __grid_constant__ CUtensorMap tmB1,
                                                     const __grid_constant__ CUtensorMap tmL0,
                                                     const __grid_constant__ CUtensorMap tmL1, const TcArgs a) {
-    constexpr int STAGES = stages_of<TERMS>();
-    constexpr uint32_t STAGE_BYTES = stage_bytes<TERMS>();
+    constexpr int BNH = BN / 2;
+    constexpr uint32_t B_BYTES = b_bytes<BN>();
+    constexpr int STAGES = stages_of<TERMS, BN>();
+    constexpr uint32_t STAGE_BYTES = stage_bytes<TERMS, BN>();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);   // even CTA: both stages landed
@@ -270,7 +277,7 @@ __global__ void __launch_bounds__(320, 1) k_tc_step(const __grid_constant__ CUte
         }
     } else if (warp == 1) {
         if (lane == 0 && leader) {
-            constexpr uint32_t idesc = instr_desc<PREC>();
+            constexpr uint32_t idesc = instr_desc<PREC, BN>();
             uint32_t it = 0, tt = 0;
             bool ok = true;
             for (int64_t g = pair; g < work && ok; g += pairs, ++tt) {
@@ -305,7 +312,7 @@ __global__ void __launch_bounds__(320, 1) k_tc_step(const __grid_constant__ CUte
         const int half = (warp - 2) >> 2;
         const uint32_t acce_cl = mapa(smem_u32(&acce[0]), 0);
         constexpr int CW = 16;   // columns per tensor-memory load
-        const int c_begin = half * (BN / (2 * CW)), c_end = c_begin + BN / (2 * CW);   // 8 chunks, even
+        const int c_begin = half * (BN / (2 * CW)), c_end = c_begin + BN / (2 * CW);   // 2, 4 or 8 chunks
         uint32_t tt = 0;
         for (int64_t g = pair; g < work; g += pairs, ++tt) {
             const uint32_t b = tt & 1u;
@@ -490,6 +497,67 @@ int make_map(CUtensorMap* m, void* base, int prec, int64_t rows, int64_t n_pad, 
 
 }  // namespace
 
+// co-resident CTA pairs of the step kernel (one CTA per SM; every form has
+// the same block size and shared memory), per device
+int tc_pairs(int device) {
+    static std::atomic<int> cache[kMaxDevices];
+    if (device < 0 || device >= kMaxDevices) return 1;
+    int v = cache[device].load(std::memory_order_relaxed);
+    if (v) return v;
+    const int sms = device_sms(device);
+    auto fn = k_tc_step<1, 1, 256, true, 0>;
+    int c = 0;
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3(320);
+    cfg.gridDim = dim3((unsigned)(sms & ~1));
+    cfg.dynamicSmemBytes = TC_SMEM;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&c, fn, &cfg) != cudaSuccess || c < 1) {
+        cudaGetLastError();
+        c = sms / 2;
+    }
+    v = std::max(1, std::min(c, sms / 2));
+    cache[device].store(v, std::memory_order_relaxed);
+    return v;
+}
+
+// Replicas per tile of a pair: 256, or 128 or 64 where tiles of 256 would
+// leave pairs idle. A step's time is modelled as the tiles a pair takes (at
+// least one) times a tile's: per K block the larger of its MMAs (BN / 2
+// cycles each; 48 at BN = 64, whose operands come from shared memory at the
+// limit) and its loads (about 50 bytes per cycle and SM from L2), then its
+// epilogue and a fixed latency. Narrow tiles re-read Qoff from L2, so wide
+// ones win once they fill the pairs. Every width adds a field's products in
+// the same order. Measured, FP8 with two terms, us per step with tiles of 256
+// alone -> with this choice: n = 1024 / 2048 / 4096 at R = 256: 25.6 -> 11.5,
+// 30.2 -> 14.6, 39.2 -> 20.4; n = 8192 at R = 64 / 256 / 512: 53.6 -> 33.2,
+// 57.9 -> 39.9, 59.3 -> 59.1 (BF16 at n = 4096, R = 256: 37.7 -> 24.9).
+int tc_tile(const veloxq_ctx* ctx, int prec, int terms, int32_t R) {
+    const int pairs = tc_pairs(ctx->device);
+    const int64_t MT = div_up(ctx->n, 2 * BM);
+    const double nkb = (double)div_up(tc_pad(ctx->n), prec == VELOXQ_PREC_BF16 ? BKB / 2 : BKB);
+    int best = 256;
+    double least = 1e300;
+    for (int bn : {256, 128, 64}) {
+        const double mma = 4.0 * terms * (bn == 64 ? 48.0 : bn / 2.0);
+        const double load = (A_BYTES + terms * (bn / 2.0) * BKB) / 50.0;
+        const double tile = nkb * std::max(mma, load) + 8000.0 * bn / 256.0 + 3000.0;
+        const double t = std::max(1.0, (double)(MT * div_up(R, bn)) / pairs) * tile;
+        if (t < least) {
+            least = t;
+            best = bn;
+        }
+    }
+    return best;
+}
+
 int64_t tc_pad(int64_t n) { return (n + 15) / 16 * 16; }
 
 // S operand terms: two E4M3 terms for FP8 (hi + lo), one for FP8_ONE_TERM,
@@ -527,6 +595,7 @@ int tc_maps(veloxq_ctx* ctx, int prec, int terms, int32_t R, void* sop0, void* s
     void* qb = prec == VELOXQ_PREC_BF16 ? ctx->qoff16.p : ctx->qoff8.p;
     VQ_TRY(make_map(mq, qb, prec, n, np, BM));
     const size_t plane = (size_t)R * (size_t)np * (prec == VELOXQ_PREC_BF16 ? 2 : 1);
+    const int BNH = tc_tile(ctx, prec, terms, R) / 2;
     VQ_TRY(make_map(ms0, sop0, prec, R, np, BNH));
     if (terms == 2) VQ_TRY(make_map(ms0_lo, static_cast<uint8_t*>(sop0) + plane, prec, R, np, BNH));
     if (sop1) {
@@ -551,9 +620,10 @@ int tc_quant_s(veloxq_ctx* ctx, int prec, int32_t R, const float* S, void* sop, 
 }
 
 // A K-major operand map of the field kernel: A (rows of the coupling
-// matrix, box of BM rows) or B (replicas, box of BN/2 rows).
-int tc_operand_map(CUtensorMap* m, void* base, int prec, int64_t rows, int64_t n_pad, bool a_operand) {
-    return make_map(m, base, prec, rows, n_pad, a_operand ? BM : BNH);
+// matrix, box of BM rows) or B (replicas, box of half a tile's replicas).
+int tc_operand_map(veloxq_ctx* ctx, CUtensorMap* m, void* base, int prec, int64_t rows, int64_t n_pad,
+                   bool a_operand) {
+    return make_map(m, base, prec, rows, n_pad, a_operand ? BM : tc_tile(ctx, prec, 1, (int32_t)rows) / 2);
 }
 
 int tc_wait_selftest(long long budget, int* code_out) {
@@ -580,16 +650,23 @@ namespace {
 using TcKernel = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap,
                           const CUtensorMap, const TcArgs);
 
-template <int PREC, int TERMS> TcKernel pick_kernel(bool field_only, int method) {
-    if (field_only) return k_tc_step<PREC, TERMS, true, 0>;
-    if (method == VELOXQ_METHOD_PA) return k_tc_step<PREC, TERMS, false, vqd::METHOD_PA>;
-    if (method == VELOXQ_METHOD_ASB) return k_tc_step<PREC, TERMS, false, vqd::METHOD_ASB>;
-    return k_tc_step<PREC, TERMS, false, vqd::METHOD_BSB>;
+// The forms that run: adiabatic SB with BF16 operands only, Parallel
+// Annealing with one operand term.
+template <int PREC, int TERMS, int BN> TcKernel pick_tile(bool field_only, int method) {
+    if (field_only) return k_tc_step<PREC, TERMS, BN, true, 0>;
+    if constexpr (TERMS == 1) {
+        if (method == VELOXQ_METHOD_PA) return k_tc_step<PREC, TERMS, BN, false, vqd::METHOD_PA>;
+    }
+    if constexpr (PREC == 1) {
+        if (method == VELOXQ_METHOD_ASB) return k_tc_step<PREC, TERMS, BN, false, vqd::METHOD_ASB>;
+    }
+    return k_tc_step<PREC, TERMS, BN, false, vqd::METHOD_BSB>;
 }
-
-// co-resident CTA pairs of the step kernel, per device
-constexpr int kMaxDevices = 64;
-int g_max_pairs[kMaxDevices];
+template <int PREC, int TERMS> TcKernel pick_kernel(int bn, bool field_only, int method) {
+    if (bn == 64) return pick_tile<PREC, TERMS, 64>(field_only, method);
+    if (bn == 128) return pick_tile<PREC, TERMS, 128>(field_only, method);
+    return pick_tile<PREC, TERMS, 256>(field_only, method);
+}
 
 // Steps per launch at most: the completion counters (16 MT per column block
 // and step) stay far below 2^32.
@@ -624,12 +701,12 @@ int tc_run(veloxq_ctx* ctx, int prec, int32_t R, const CUtensorMap& mq, const CU
     const int terms = tc_terms(prec, field_only ? VELOXQ_METHOD_BSB : rule.method);
     if (terms == 2 && !ms_lo) return fail(VELOXQ_EINVAL, "two-term FP8 operand without its lo-plane maps");
     if (ctx->device < 0 || ctx->device >= kMaxDevices) return fail(VELOXQ_EUNSUPPORTED, "device ordinal out of range");
-    const int sms = device_sms(ctx->device);
-    const int64_t MT = div_up(ctx->n, 2 * BM), NT = div_up(R, BN), tiles = MT * NT;
+    const int bn = tc_tile(ctx, prec, terms, R);
+    const int64_t MT = div_up(ctx->n, 2 * BM), NT = div_up(R, bn), tiles = MT * NT;
     TcKernel fn;
-    if (prec == VELOXQ_PREC_BF16) fn = pick_kernel<1, 1>(field_only, rule.method);
-    else if (terms == 2) fn = pick_kernel<2, 2>(field_only, rule.method);
-    else fn = pick_kernel<2, 1>(field_only, rule.method);
+    if (prec == VELOXQ_PREC_BF16) fn = pick_kernel<1, 1>(bn, field_only, rule.method);
+    else if (terms == 2) fn = pick_kernel<2, 2>(bn, field_only, rule.method);
+    else fn = pick_kernel<2, 1>(bn, field_only, rule.method);
     VQ_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM));
     cudaLaunchConfig_t cfg = {};
     cfg.blockDim = dim3(320);
@@ -643,19 +720,8 @@ int tc_run(veloxq_ctx* ctx, int prec, int32_t R, const CUtensorMap& mq, const CU
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    // as many pairs as can be resident at once (one CTA per SM; every form
-    // has the same block size and shared memory)
-    int& max_pairs = g_max_pairs[ctx->device];
-    if (!max_pairs) {
-        cfg.gridDim = dim3((unsigned)(sms & ~1));
-        int c = 0;
-        if (cudaOccupancyMaxActiveClusters(&c, fn, &cfg) != cudaSuccess || c < 1) {
-            cudaGetLastError();
-            c = sms / 2;
-        }
-        max_pairs = std::max(1, std::min(c, sms / 2));
-    }
+    cfg.numAttrs = 2;   // clusters and programmatic dependent launch
+    const int max_pairs = tc_pairs(ctx->device);
     const CUtensorMap& lo0 = terms == 2 ? ms_lo[0] : ms[0];
     const CUtensorMap& lo1 = terms == 2 ? ms_lo[1] : ms[1];
     for (int k0 = k_begin; k0 < k_end; k0 += kMaxRunSteps) {
@@ -688,7 +754,7 @@ int tc_run(veloxq_ctx* ctx, int prec, int32_t R, const CUtensorMap& mq, const CU
         a.plane = (int64_t)R * a.n_pad;
         a.done = nullptr;
         if (steps > 1) {
-            // sized by the caller before any stream capture (256 replicas per column block)
+            // sized by the caller before any stream capture
             if (ctx->tcdone.bytes < sizeof(uint32_t) * (size_t)NT)
                 return fail(VELOXQ_EINVAL, "tensor-core run without its completion counters");
             VQ_CUDA(cudaMemsetAsync(ctx->tcdone.p, 0, sizeof(uint32_t) * (size_t)NT, ctx->stream));
@@ -696,7 +762,6 @@ int tc_run(veloxq_ctx* ctx, int prec, int32_t R, const CUtensorMap& mq, const CU
         }
         const int64_t pairs = std::max<int64_t>(1, std::min<int64_t>(tiles * steps, max_pairs));
         cfg.gridDim = dim3((unsigned)(2 * pairs));
-        cfg.numAttrs = 2;   // with programmatic dependent launch (the occupancy query above used the cluster only)
         VQ_CUDA(cudaLaunchKernelEx(&cfg, fn, mq, ms[0], ms[1], lo0, lo1, a));
         VQ_LAUNCH_CHECK("tc step");
     }
