@@ -194,7 +194,10 @@ int launch_step(veloxq_ctx* ctx, int32_t R, const float* S_cur, float* S_nxt, co
         else if (unroll == 4) VQ_STEP_U(VV, WT, WPTR, SC, 4);       \
         else VQ_STEP_U(VV, WT, WPTR, SC, 1);                        \
     } while (0)
-    const int unroll = (ctx->stream_unroll == 6 && ctx->uniform_deg == 6) ? 6 : ctx->stream_unroll == 4 ? 4 : 1;
+    // without a timing trial (single steps and fields): six at once on rows of exactly six couplings, where it is
+    // the form every trial picks (cubic lattice L = 100, 256 replicas: 0.70 ms against 0.80 one at a time)
+    const bool six = ctx->uniform_deg == 6 && (ctx->stream_unroll == 6 || ctx->stream_unroll == 0);
+    const int unroll = six ? 6 : ctx->stream_unroll == 4 ? 4 : 1;
     if (ctx->w8.p) {
         const int8_t* w = ctx->w8.as<int8_t>();
         if (V == 4) VQ_STEP(4, int8_t, w, 0.5f); else if (V == 2) VQ_STEP(2, int8_t, w, 0.5f); else VQ_STEP(1, int8_t, w, 0.5f);
