@@ -157,8 +157,8 @@ typedef struct {
 
 /* Device timing of the last veloxq_solve or veloxq_grad on a context, from
  * CUDA events recorded on the stream the kernels run on. For veloxq_grad,
- * ms_main is the reverse sweep (the adjoint step kernels, 3 launches per
- * step) and path is VELOXQ_PATH_STREAM. */
+ * ms_main is the reverse sweep (the adjoint step kernels, 2 launches per
+ * step and one more for the sums of up to 32 steps) and path is VELOXQ_PATH_STREAM. */
 typedef struct {
     double ms_total;        /* first to last kernel of the solve (or gradient) */
     double ms_main;         /* the integration: the resident kernel, or the captured steps up to the last one */

@@ -16,6 +16,7 @@
 // Forward states are kept every C steps; each segment is recomputed forward
 // (bit-identical: the same kernels) before its reverse sweep, so the wall
 // masks of the reverse sweep are those of the forward run.
+#include <algorithm>
 #include <cmath>
 #include <vector>
 
@@ -165,20 +166,24 @@ __global__ void __launch_bounds__(kAdjThreads, UNROLL == 6 ? 8 : 1) k_adj_b(int6
     vqd::vstore<V>(lam_s + me, g);
 }
 
-// acc[0] += dL/ddt, acc[1] += dL/dc0, acc[2 + k] = dL/da_k (fixed order)
-__global__ void k_adj_reduce(const double* __restrict__ parts3, int G, int k, double* acc) {
+// The sums of `gridDim.x` reverse steps, step k0 - blockIdx.x from its own
+// parts: acc[k] = dL/ddt, acc[K + k] = dL/dc0, acc[2 K + k] = dL/da_k of step k
+// (fixed order).
+__global__ void k_adj_reduce(const double* __restrict__ parts3, int G, int k0, int K, double* acc) {
     __shared__ double sh[3 * kAdjThreads];
+    const double* p3 = parts3 + (size_t)blockIdx.x * 3 * G;
+    const int k = k0 - (int)blockIdx.x;
     double v[3] = {0.0, 0.0, 0.0};
     for (int g = threadIdx.x; g < G; g += blockDim.x) {
-        v[0] += parts3[3 * g];
-        v[1] += parts3[3 * g + 1];
-        v[2] += parts3[3 * g + 2];
+        v[0] += p3[3 * g];
+        v[1] += p3[3 * g + 1];
+        v[2] += p3[3 * g + 2];
     }
     block_sum<3>(v, sh);
     if (threadIdx.x == 0) {
-        acc[0] += v[0];
-        acc[1] += v[1];
-        acc[2 + k] = v[2];
+        acc[k] = v[0];
+        acc[(size_t)K + k] = v[1];
+        acc[2 * (size_t)K + k] = v[2];
     }
 }
 
@@ -190,9 +195,19 @@ __global__ void k_adj_loss_total(const double* __restrict__ parts, int G, double
     if (threadIdx.x == 0) *out = v[0];
 }
 
-// dL/dknot_j = sum_k w_kj dL/da_k, with the interpolation weights of the schedule.
-__global__ void k_adj_knots(int K, int nk, const double* __restrict__ da, double* dknots) {
+// dL/dknot_j = sum_k w_kj dL/da_k, with the interpolation weights of the
+// schedule; threads 64 and 65 add dL/ddt and dL/dc0 of the steps, last step
+// first, into tot[0] and tot[1].
+__global__ void k_adj_knots(int K, int nk, const double* __restrict__ acc, double* dknots, double* tot) {
     const int j = threadIdx.x;
+    if (j >= 64) {
+        if (j > 65) return;
+        double s = 0.0;
+        for (int k = K - 1; k >= 0; --k) s += acc[(size_t)(j - 64) * K + k];
+        tot[j - 64] = s;
+        return;
+    }
+    const double* da = acc + 2 * (size_t)K;
     if (j >= nk) return;
     double s = 0.0;
     for (int k = 0; k < K; ++k) {
@@ -283,23 +298,27 @@ int adjoint_run(veloxq_ctx* ctx, int32_t R, const RunParams& p, const std::vecto
     const int M = (int)div_up(K, C);                  // checkpoints: states before steps 0, C, 2C, ...
     const int V = vec_width(R);
     const size_t blk = sizeof(float) * (size_t)nR;
-    // checkpoints (S, Y) x M, segment states (S, Y) x C, 3 adjoint blocks
+    // checkpoints (S, Y) x M, states (S, Y) of a segment after its first .. C-th step, 3 adjoint blocks; the
+    // per-step sums are reduced for up to kSumSteps reverse steps at a time
+    constexpr int kSumSteps = 32;
     DevBuf ck, seg, adj, red;
     VQ_TRY(ck.ensure(2 * blk * (size_t)M));
-    VQ_TRY(seg.ensure(2 * blk * (size_t)(C + 1)));
+    VQ_TRY(seg.ensure(2 * blk * (size_t)std::min(C, K)));
     VQ_TRY(adj.ensure(3 * blk));
-    VQ_TRY(red.ensure(sizeof(double) * (size_t)(3 * kAdjBlocks + kAdjBlocks + 2 + K + 8 + n_knots)));
+    VQ_TRY(red.ensure(sizeof(double) * (size_t)(3 * kAdjBlocks * (size_t)std::min(C, kSumSteps) + kAdjBlocks +
+                                                3 * (size_t)K + 8 + n_knots)));
     auto ckS = [&](int m) { return ck.as<float>() + (size_t)(2 * m) * nR; };
     auto ckY = [&](int m) { return ck.as<float>() + (size_t)(2 * m + 1) * nR; };
-    auto sgS = [&](int t) { return seg.as<float>() + (size_t)(2 * t) * nR; };
-    auto sgY = [&](int t) { return seg.as<float>() + (size_t)(2 * t + 1) * nR; };
+    // state of segment m before its step t: the checkpoint, or segment state t
+    auto sgS = [&](int m, int t) { return t == 0 ? ckS(m) : seg.as<float>() + (size_t)(2 * (t - 1)) * nR; };
+    auto sgY = [&](int m, int t) { return t == 0 ? ckY(m) : seg.as<float>() + (size_t)(2 * (t - 1) + 1) * nR; };
     float* lam_s = adj.as<float>();
     float* lam_y = lam_s + nR;
     float* gsl = lam_y + nR;
     double* parts3 = red.as<double>();
-    double* parts = parts3 + 3 * kAdjBlocks;
-    double* acc = parts + kAdjBlocks;                  // [0] ddt [1] dc0 [2..2+K) da_k
-    double* lossd = acc + 2 + K;
+    double* parts = parts3 + 3 * (size_t)kAdjBlocks * std::min(C, kSumSteps);
+    double* acc = parts + kAdjBlocks;                  // per step: [0..K) ddt, [K..2K) dc0, [2K..3K) da_k
+    double* lossd = acc + 3 * (size_t)K;               // [0] loss, [1] ddt, [2] dc0
     double* dkn = lossd + 8;
     const float* at = ctx->a_table.as<float>();
     cudaStream_t st = ctx->stream;
@@ -314,21 +333,20 @@ int adjoint_run(veloxq_ctx* ctx, int32_t R, const RunParams& p, const std::vecto
     ev.e.assign((size_t)(2 + 2 * M), nullptr);
     for (cudaEvent_t& x : ev.e) VQ_CUDA(cudaEventCreate(&x));
     VQ_CUDA(cudaEventRecord(ev.e[0], st));
-    int64_t launches = 0;
-    VQ_CUDA(cudaMemsetAsync(acc, 0, sizeof(double) * (size_t)(2 + K), st));
+    int64_t launches = 0, reverse = 0;
 
-    // ---- forward with checkpoints (two working buffers in seg[0], seg[1]) ----
-    VQ_TRY(launch_init_state(ctx, R, seed, p.sigma0, LAYOUT_NR, sgS(0), sgY(0)));
-    float* cS = sgS(0);
-    float* cY = sgY(0);
-    float* nS = sgS(1);
+    // ---- forward: every C-th state goes straight to its checkpoint, the last segment's states to where the
+    // reverse sweep reads them; the others alternate between two segment states ----
+    VQ_TRY(launch_init_state(ctx, R, seed, p.sigma0, LAYOUT_NR, ckS(0), ckY(0)));
+    float *cS = ckS(0), *cY = ckY(0);
     for (int k = 0; k < K; ++k) {
-        if (k % C == 0) {
-            VQ_CUDA(cudaMemcpyAsync(ckS(k / C), cS, blk, cudaMemcpyDeviceToDevice, st));
-            VQ_CUDA(cudaMemcpyAsync(ckY(k / C), cY, blk, cudaMemcpyDeviceToDevice, st));
-        }
-        VQ_TRY(stream_step_y(ctx, R, cS, nS, cY, cY, at, k, p.dt, p.a0, p.c0, nullptr));
-        std::swap(cS, nS);
+        const int m = k / C, t = k - m * C;
+        const bool to_ck = t == C - 1 && m + 1 < M;
+        float* nS = to_ck ? ckS(m + 1) : sgS(m, m == M - 1 ? t + 1 : 1 + (t & 1));
+        float* nY = to_ck ? ckY(m + 1) : sgY(m, m == M - 1 ? t + 1 : 1);
+        VQ_TRY(stream_step_y(ctx, R, cS, nS, cY, nY, at, k, p.dt, p.a0, p.c0, nullptr));
+        cS = nS;
+        cY = nY;
     }
     launches += 1 + K + 2;   // init, forward steps, loss and its total
     // ---- loss and seed ----
@@ -340,32 +358,40 @@ int adjoint_run(veloxq_ctx* ctx, int32_t R, const RunParams& p, const std::vecto
     // ---- reverse sweep, one segment at a time ----
     for (int m = M - 1; m >= 0; --m) {
         const int k0 = m * C, k1 = std::min(K, k0 + C);
-        // recompute the segment: state t (before step k0 + t) into seg[t]
-        VQ_CUDA(cudaMemcpyAsync(sgS(0), ckS(m), blk, cudaMemcpyDeviceToDevice, st));
-        VQ_CUDA(cudaMemcpyAsync(sgY(0), ckY(m), blk, cudaMemcpyDeviceToDevice, st));
-        for (int t = 0; t < k1 - k0 - 1; ++t)
-            VQ_TRY(stream_step_y(ctx, R, sgS(t), sgS(t + 1), sgY(t), sgY(t + 1), at, k0 + t, p.dt, p.a0, p.c0, nullptr));
-        launches += k1 - k0 - 1 + 3 * (k1 - k0);
+        // recompute the segment's states (the forward run left the last segment's)
+        const int again = m == M - 1 ? 0 : k1 - k0 - 1;
+        for (int t = 0; t < again; ++t)
+            VQ_TRY(stream_step_y(ctx, R, sgS(m, t), sgS(m, t + 1), sgY(m, t), sgY(m, t + 1), at, k0 + t, p.dt, p.a0,
+                                 p.c0, nullptr));
+        launches += again + 2 * (k1 - k0);
         VQ_CUDA(cudaEventRecord(ev.e[2 + 2 * m], st));
+        int waiting = 0;   // reverse steps whose sums are in parts3
         for (int k = k1 - 1; k >= k0; --k) {
             const int t = k - k0;
+            double* p3 = parts3 + 3 * (size_t)kAdjBlocks * waiting;
             if (ctx->w8.p)
-                VQ_TRY(adj_dispatch_step<int8_t>(ctx, V, R, ctx->w8.as<int8_t>(), 0.5f, sgS(t), sgY(t), a_host[k], p.dt,
-                                                 p.a0, p.c0, lam_s, lam_y, gsl, parts3));
+                VQ_TRY(adj_dispatch_step<int8_t>(ctx, V, R, ctx->w8.as<int8_t>(), 0.5f, sgS(m, t), sgY(m, t), a_host[k],
+                                                 p.dt, p.a0, p.c0, lam_s, lam_y, gsl, p3));
             else
-                VQ_TRY(adj_dispatch_step<float>(ctx, V, R, ctx->wf.as<float>(), 1.0f, sgS(t), sgY(t), a_host[k], p.dt,
-                                                p.a0, p.c0, lam_s, lam_y, gsl, parts3));
-            k_adj_reduce<<<1, kAdjThreads, 0, st>>>(parts3, kAdjBlocks, k, acc);
-            VQ_LAUNCH_CHECK("adjoint reduce");
+                VQ_TRY(adj_dispatch_step<float>(ctx, V, R, ctx->wf.as<float>(), 1.0f, sgS(m, t), sgY(m, t), a_host[k],
+                                                p.dt, p.a0, p.c0, lam_s, lam_y, gsl, p3));
+            if (++waiting == std::min(C, kSumSteps) || k == k0) {
+                k_adj_reduce<<<waiting, kAdjThreads, 0, st>>>(parts3, kAdjBlocks, k + waiting - 1, K, acc);
+                VQ_LAUNCH_CHECK("adjoint reduce");
+                waiting = 0;
+                ++launches;
+                ++reverse;
+            }
         }
+        reverse += 2 * (k1 - k0);
         VQ_CUDA(cudaEventRecord(ev.e[3 + 2 * m], st));
     }
-    k_adj_knots<<<1, 64, 0, st>>>(K, n_knots, acc + 2, dkn);
+    k_adj_knots<<<1, 96, 0, st>>>(K, n_knots, acc, dkn, lossd + 1);
     VQ_LAUNCH_CHECK("adjoint knots");
     launches += 1;
     VQ_CUDA(cudaEventRecord(ev.e[1], st));
-    std::vector<double> h((size_t)(2 + K + 8 + n_knots));
-    VQ_CUDA(cudaMemcpyAsync(h.data(), acc, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, st));
+    std::vector<double> h((size_t)(8 + n_knots));
+    VQ_CUDA(cudaMemcpyAsync(h.data(), lossd, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, st));
     VQ_CUDA(cudaStreamSynchronize(st));
     if (tm) {
         VQ_CUDA(cudaEventElapsedTime(&tm->ms_total, ev.e[0], ev.e[1]));
@@ -376,13 +402,13 @@ int adjoint_run(veloxq_ctx* ctx, int32_t R, const RunParams& p, const std::vecto
             tm->ms_reverse += x;
         }
         tm->launches = launches;
-        tm->reverse_launches = 3 * (int64_t)K;
+        tm->reverse_launches = reverse;
     }
-    if (loss) *loss = ctx->K0 + h[2 + K] / (double)R;
-    if (d_dt) *d_dt = h[0];
-    if (d_c0) *d_c0 = h[1];
+    if (loss) *loss = ctx->K0 + h[0] / (double)R;
+    if (d_dt) *d_dt = h[1];
+    if (d_c0) *d_c0 = h[2];
     if (d_knots)
-        for (int j = 0; j < n_knots; ++j) d_knots[j] = h[2 + K + 8 + j];
+        for (int j = 0; j < n_knots; ++j) d_knots[j] = h[8 + j];
     return VELOXQ_OK;
 }
 
