@@ -168,7 +168,7 @@ struct CtxExtra {
     // scratch of a batched launch headed by this context (instance table,
     // per-instance results, error word): owned here, so that batches headed
     // by different contexts never share it
-    DevBuf bwork, bbest, berr;
+    DevBuf bwork, bbest, berr, bx;
     int tune_stages = 0, tune_split = 0;   // form of the last batched launch headed by this context
     BatchGraph bgraph;                     // its captured device part
     ~CtxExtra() {
@@ -257,10 +257,15 @@ std::vector<float> schedule_table(const RunParams& p) {
 
 int upload_schedule(veloxq_ctx* ctx, const RunParams& p) {
     std::vector<float> a = schedule_table(p);
+    if (ctx->a_table.p && a.size() == ctx->a_host.size() &&
+        std::memcmp(a.data(), ctx->a_host.data(), sizeof(float) * a.size()) == 0)
+        return VELOXQ_OK;   // the device holds these values
+    ctx->a_host.clear();
     VQ_TRY(ctx->a_table.ensure(sizeof(float) * a.size()));
     VQ_CUDA(cudaMemcpyAsync(ctx->a_table.p, a.data(), sizeof(float) * a.size(), cudaMemcpyHostToDevice, ctx->stream));
     // the host vector dies at return: make the copy complete first
     VQ_CUDA(cudaStreamSynchronize(ctx->stream));
+    ctx->a_host = std::move(a);
     return VELOXQ_OK;
 }
 
@@ -462,11 +467,10 @@ int enqueue_loop(veloxq_ctx* ctx, veloxq_path path, int32_t R, const RunParams& 
         int64_t* parts = ctx->ework.as<int64_t>();
         if (path == VELOXQ_PATH_DENSE) VQ_TRY(dense_energy(ctx, R, cur, parts, &np, tc_energy));
         else VQ_TRY(stream_energy(ctx, R, cur, parts, &np));
-        VQ_TRY(launch_best_update(ctx, R, np, parts, ctx->best_e.as<int64_t>(), ctx->flags.as<uint8_t>()));
+        VQ_TRY(launch_best_update(ctx, R, np, parts, ctx->res_best(), ctx->flags.as<uint8_t>()));
         VQ_TRY(launch_best_bits(ctx, R, lay, cur, ctx->flags.as<uint8_t>(), ctx->best_bits.as<uint32_t>()));
     }
-    VQ_TRY(launch_argmin_unpack(ctx, R, ctx->best_e.as<int64_t>(), ctx->best_bits.as<uint32_t>(),
-                                ctx->misc.as<int64_t>(), ctx->xout.as<uint8_t>()));
+    VQ_TRY(launch_argmin_unpack(ctx, R, ctx->res_best(), ctx->best_bits.as<uint32_t>(), ctx->res_win(), ctx->res_x(R)));
     return VELOXQ_OK;
 }
 
@@ -663,21 +667,19 @@ int veloxq_solve(veloxq_ctx* ctx, int32_t replicas, int32_t steps, const veloxq_
     int64_t launches = 0;
 
     VQ_TRY(upload_schedule(ctx, p));
-    VQ_TRY(ctx->best_e.ensure(sizeof(int64_t) * R));
     VQ_TRY(ctx->best_bits.ensure(sizeof(uint32_t) * R * nw));
-    VQ_TRY(ctx->misc.ensure(sizeof(int64_t) * 16));
-    VQ_TRY(ctx->xout.ensure((size_t)n));
-    int32_t main_launches = 1;
+    VQ_TRY(ctx->res.ensure(sizeof(int64_t) * (size_t)(2 + R) + (size_t)n));
+    int32_t main_launches = 1, window = 0;
     if (path == VELOXQ_PATH_RESIDENT) {
         VQ_CUDA(cudaEventRecord(ex->t0, ctx->stream));
         VQ_CUDA(cudaEventRecord(ex->t1, ctx->stream));
         VQ_TRY(resident_run(ctx, replicas, p, seed, 0, steps, nullptr, nullptr, nullptr, nullptr, nullptr,
-                            ctx->best_e.as<int64_t>(), ctx->best_bits.as<uint32_t>()));
+                            ctx->res_best(), ctx->best_bits.as<uint32_t>()));
         VQ_CUDA(cudaEventRecord(ex->t2, ctx->stream));
-        VQ_TRY(launch_argmin_unpack(ctx, replicas, ctx->best_e.as<int64_t>(), ctx->best_bits.as<uint32_t>(),
-                                    ctx->misc.as<int64_t>(), ctx->xout.as<uint8_t>()));
+        VQ_TRY(launch_argmin_unpack(ctx, replicas, ctx->res_best(), ctx->best_bits.as<uint32_t>(), ctx->res_win(),
+                                    ctx->res_x(R)));
         VQ_CUDA(cudaEventRecord(ex->t3, ctx->stream));
-        launches = 3;
+        launches = 2;
     } else {
         const Layout lay = path == VELOXQ_PATH_DENSE ? LAYOUT_RN : LAYOUT_NR;
         const int nparts = stream_energy_parts_count(ctx, path, replicas);
@@ -706,7 +708,7 @@ int veloxq_solve(veloxq_ctx* ctx, int32_t replicas, int32_t steps, const veloxq_
         if (use_tc || tc_e) VQ_CUDA(cudaMemsetAsync(ctx->errw.p, 0, sizeof(int), ctx->stream));
         if (use_tc) VQ_TRY(tc_quant_s(ctx, p.prec, replicas, ctx->s_a.as<float>(), tc.sop[0], rule_of(p)));
         if (use_t32) VQ_TRY(t32_split(ctx, replicas, ctx->s_a.as<float>(), rule_of(p), false, &t32r));
-        VQ_CUDA(cudaMemsetAsync(ctx->best_e.p, 0x7f, sizeof(int64_t) * R, ctx->stream));
+        VQ_CUDA(cudaMemsetAsync(ctx->res_best(), 0x7f, sizeof(int64_t) * R, ctx->stream));
         VQ_CUDA(cudaMemsetAsync(ctx->best_bits.p, 0, sizeof(uint32_t) * R * nw, ctx->stream));
         // the captured loop depends on every pointer and parameter below
         std::vector<uint64_t> key = {(uint64_t)path, (uint64_t)p.prec, (uint64_t)(uintptr_t)ctx->sop_a.p,
@@ -714,9 +716,8 @@ int veloxq_solve(veloxq_ctx* ctx, int32_t replicas, int32_t steps, const veloxq_
                                      (uint64_t)R, (uint64_t)steps, (uint64_t)p.readout_every,
                                      (uint64_t)(uintptr_t)ctx->s_a.p, (uint64_t)(uintptr_t)ctx->s_b.p,
                                      (uint64_t)(uintptr_t)ctx->y.p, (uint64_t)(uintptr_t)ctx->ework.p,
-                                     (uint64_t)(uintptr_t)ctx->best_e.p, (uint64_t)(uintptr_t)ctx->best_bits.p,
-                                     (uint64_t)(uintptr_t)ctx->flags.p, (uint64_t)(uintptr_t)ctx->misc.p,
-                                     (uint64_t)(uintptr_t)ctx->xout.p, (uint64_t)(uintptr_t)ctx->a_table.p};
+                                     (uint64_t)(uintptr_t)ctx->res.p, (uint64_t)(uintptr_t)ctx->best_bits.p,
+                                     (uint64_t)(uintptr_t)ctx->flags.p, (uint64_t)(uintptr_t)ctx->a_table.p};
         key.push_back((uint64_t)p.method);
         for (uint64_t v : {(uint64_t)tc_e, (uint64_t)ctx->eplanes, (uint64_t)(uintptr_t)ctx->eplane.p,
                            (uint64_t)(uintptr_t)ctx->exop.p, (uint64_t)(uintptr_t)ctx->efield.p,
@@ -776,11 +777,14 @@ int veloxq_solve(veloxq_ctx* ctx, int32_t replicas, int32_t steps, const veloxq_
         }
         if (use_tc || tc_e) VQ_TRY(check_err_word(ctx));
     }
-    std::vector<int64_t> be((size_t)R);
-    int64_t misc[2] = {0, 0};
-    VQ_CUDA(cudaMemcpyAsync(be.data(), ctx->best_e.p, sizeof(int64_t) * R, cudaMemcpyDeviceToHost, ctx->stream));
-    VQ_CUDA(cudaMemcpyAsync(misc, ctx->misc.p, sizeof(misc), cudaMemcpyDeviceToHost, ctx->stream));
-    if (x_best) VQ_CUDA(cudaMemcpyAsync(x_best, ctx->xout.p, (size_t)n, cudaMemcpyDeviceToHost, ctx->stream));
+    // one copy brings the results back; a long vector goes straight to the caller
+    const bool direct = n > (1 << 18);
+    const size_t head = sizeof(int64_t) * (size_t)(2 + R);
+    std::vector<int64_t> host((head + (x_best && !direct ? (size_t)n : 0) + 7) / 8);
+    VQ_CUDA(cudaMemcpyAsync(host.data(), ctx->res.p, head + (x_best && !direct ? (size_t)n : 0), cudaMemcpyDeviceToHost,
+                            ctx->stream));
+    if (x_best && direct)
+        VQ_CUDA(cudaMemcpyAsync(x_best, ctx->res_x(R), (size_t)n, cudaMemcpyDeviceToHost, ctx->stream));
     VQ_CUDA(cudaStreamSynchronize(ctx->stream));
     VQ_LAUNCH_CHECK("solve");
     VQ_TRY(t32_check(ctx));
@@ -801,10 +805,11 @@ int veloxq_solve(veloxq_ctx* ctx, int32_t replicas, int32_t steps, const veloxq_
         ex->timed = true;
     }
     const int sh = ctx->energy_shift;
-    if (E_best) *E_best = std::ldexp((double)misc[1], -sh);
-    if (E_best_int) *E_best_int = misc[1] >> sh;
+    if (x_best && !direct) std::memcpy(x_best, host.data() + 2 + R, (size_t)n);
+    if (E_best) *E_best = std::ldexp((double)host[1], -sh);
+    if (E_best_int) *E_best_int = host[1] >> sh;
     if (E_per_replica)
-        for (int64_t r = 0; r < R; ++r) E_per_replica[r] = std::ldexp((double)be[r], -sh);
+        for (int64_t r = 0; r < R; ++r) E_per_replica[r] = std::ldexp((double)host[2 + r], -sh);
     return VELOXQ_OK;
 }
 
@@ -841,9 +846,13 @@ int veloxq_solve_batch(veloxq_ctx* const* ctxs, int32_t count, int32_t replicas,
     CtxExtra* ex = extra(c0);
     cudaStream_t st = ex->work;
     for (int32_t m = 0; m < count; ++m) {
+        if (m > 0 && ctxs[m]->stream == ctxs[m - 1]->stream) continue;   // ordered already
         VQ_CUDA(cudaEventRecord(ex->ev, ctxs[m]->stream));
         VQ_CUDA(cudaStreamWaitEvent(st, ex->ev, 0));
     }
+    size_t xbytes = 0;
+    for (int32_t m = 0; m < count; ++m) xbytes += (size_t)ctxs[m]->n;
+    VQ_TRY(ex->bx.ensure(xbytes));
     {
         cudaStream_t keep = c0->stream;
         c0->stream = st;
@@ -888,7 +897,7 @@ int veloxq_solve_batch(veloxq_ctx* const* ctxs, int32_t count, int32_t replicas,
                 if (!batch_stages_fit(p.prec, p.method, cand, replicas / sp)) continue;
                 float ms = 0.f;
                 VQ_TRY(batch_run(ctxs, count, replicas, probe, seed, st, cand, sp, work, best_all.as<int64_t>(),
-                                 errw.as<int>(), &ms));
+                                 ex->bx.as<uint8_t>(), errw.as<int>(), &ms));
                 if (ms < best_ms) {
                     best_ms = ms;
                     stages = cand;
@@ -903,16 +912,24 @@ int veloxq_solve_batch(veloxq_ctx* const* ctxs, int32_t count, int32_t replicas,
     ex->tune_split = split;
     float ms_main = 0.f;
     int64_t nlaunch = 0;
-    VQ_TRY(batch_run(ctxs, count, replicas, p, seed, st, stages, split, work, best_all.as<int64_t>(), errw.as<int>(),
-                     &ms_main, &nlaunch, &ex->bgraph));
+    VQ_TRY(batch_run(ctxs, count, replicas, p, seed, st, stages, split, work, best_all.as<int64_t>(),
+                     ex->bx.as<uint8_t>(), errw.as<int>(), &ms_main, &nlaunch, &ex->bgraph));
     int herr = 0;
     std::vector<int64_t> h((size_t)(2 * count));
     VQ_CUDA(cudaMemcpyAsync(&herr, errw.p, sizeof(int), cudaMemcpyDeviceToHost, st));
     VQ_CUDA(cudaMemcpyAsync(h.data(), best_all.p, sizeof(int64_t) * h.size(), cudaMemcpyDeviceToHost, st));
-    for (int32_t m = 0; m < count; ++m)
-        if (x_best && x_best[m])
-            VQ_CUDA(cudaMemcpyAsync(x_best[m], ctxs[m]->xout.p, (size_t)ctxs[m]->n, cudaMemcpyDeviceToHost, st));
+    // every vector in one copy (256 copies of about a kilobyte took 4 ms)
+    std::vector<uint8_t> hx;
+    if (x_best) {
+        hx.resize(xbytes);
+        VQ_CUDA(cudaMemcpyAsync(hx.data(), ex->bx.p, xbytes, cudaMemcpyDeviceToHost, st));
+    }
     VQ_CUDA(cudaStreamSynchronize(st));
+    if (x_best) {
+        const uint8_t* at = hx.data();
+        for (int32_t m = 0; m < count; at += ctxs[m]->n, ++m)
+            if (x_best[m]) std::memcpy(x_best[m], at, (size_t)ctxs[m]->n);
+    }
     if (herr) return fail(VELOXQ_ETIMEDOUT, "a bounded wait in the batched kernel gave up (code " + std::to_string(herr) + ")");
     if (E_best)
         for (int32_t m = 0; m < count; ++m) E_best[m] = std::ldexp((double)h[2 * m + 1], -ctxs[m]->energy_shift);
@@ -1053,8 +1070,11 @@ int veloxq_steps_dev(veloxq_ctx* ctx, int32_t R, int32_t k_begin, int32_t k_coun
         VQ_TRY(t32_prepare(ctx, R, &t32));
         if (t32) VQ_TRY(t32_split(ctx, R, S, rule_of(p), true, &t32r));
     }
-    VQ_TRY(upload_schedule(ctx, p));   // waits for the stream, so for the range check of the split too
-    if (t32 && t32_bad(ctx, t32r)) t32 = false;
+    VQ_TRY(upload_schedule(ctx, p));
+    if (t32) {
+        VQ_CUDA(cudaStreamSynchronize(ctx->stream));   // the range check of the split
+        if (t32_bad(ctx, t32r)) t32 = false;
+    }
     if (path == VELOXQ_PATH_RESIDENT)
         return resident_run(ctx, R, p, 0, k_begin, k_end, S, Y, S, Y, F_last, nullptr, nullptr);
     VQ_TRY(ctx->s_b.ensure(sizeof(float) * nR));

@@ -574,7 +574,7 @@ bool batch_supported(veloxq_ctx* const* ctxs, int32_t count, int32_t R, const Ru
 // the argmin of every instance; without `graph` only the kernel, timed (the
 // autotuner's probes). stages: 4 (two CTAs per SM) or 6 (one).
 int batch_run(veloxq_ctx* const* ctxs, int32_t count, int32_t R, const RunParams& p, uint64_t seed, cudaStream_t st,
-              int stages, int split, DevBuf& work, int64_t* d_best_all, int* d_err, float* ms_main,
+              int stages, int split, DevBuf& work, int64_t* d_best_all, uint8_t* d_x, int* d_err, float* ms_main,
               int64_t* launches, BatchGraph* graph) {
     int64_t nl = 0;
     std::vector<std::pair<void*, size_t>> zero;   // operand buffers whose padding is zeroed
@@ -622,10 +622,10 @@ int batch_run(veloxq_ctx* const* ctxs, int32_t count, int32_t R, const RunParams
         VQ_TRY(c->sop_a.ensure(sopb));
         VQ_TRY(c->sop_b.ensure(sopb));
         // the K padding of the operand tiles is never written: zero it when the
-        // buffers last held another layout (or were just allocated); a captured
-        // launch zeroes it on every replay
+        // buffers last held another layout (or were just allocated), outside the
+        // captured part
         const int64_t tag = ((int64_t)R << 16) | ((int64_t)p.prec << 8) | ((int64_t)terms << 4) | 1;
-        if (graph || c->sop_tag != tag || c->sop_a.p != pa || c->sop_b.p != pb) {
+        if (c->sop_tag != tag || c->sop_a.p != pa || c->sop_b.p != pb) {
             zero.push_back({c->sop_a.p, sopb});
             zero.push_back({c->sop_b.p, sopb});
             c->sop_tag = tag;
@@ -678,9 +678,9 @@ int batch_run(veloxq_ctx* const* ctxs, int32_t count, int32_t R, const RunParams
         veloxq_ctx* c = ctxs[m];
         const int tiles = (int)div_up(c->n, emma::TI);
         VQ_TRY(c->ework.ensure(sizeof(int64_t) * (size_t)tiles * R));
-        VQ_TRY(c->xout.ensure((size_t)c->n));
         rd[m] = ReadInst{c->qx.p, c->dfix.as<int64_t>(), c->s_a.as<float>(), c->ework.as<int64_t>(),
-                         c->xout.as<uint8_t>(), (int32_t)c->n, c->energy_shift};
+                         d_x, (int32_t)c->n, c->energy_shift};
+        d_x += c->n;
         const int t = (int)c->qx_type;
         if (t < 0 || t > 3) return fail(VELOXQ_EINVAL, "unknown coupling type");
         for (int l = 0; l < tiles * (int)div_up(R, etr); ++l) {
@@ -742,12 +742,11 @@ int batch_run(veloxq_ctx* const* ctxs, int32_t count, int32_t R, const RunParams
         VQ_CUDA(cudaEventCreate(&e0));
         VQ_CUDA(cudaEventCreate(&e1));
     }
-    // the device part of the solve: operand padding, the persistent kernel
-    // between two timing events, and the final readout (one energy launch per
+    for (const auto& z : zero) VQ_CUDA(cudaMemsetAsync(z.first, 0, z.second, st));
+    // the device part of the solve: the persistent kernel between two timing events, and the final readout (one energy launch per
     // element type of Q in the batch, one finish launch)
     auto enqueue = [&]() -> int {
         const unsigned flags = graph ? cudaEventRecordExternal : cudaEventRecordDefault;
-        for (const auto& z : zero) VQ_CUDA(cudaMemsetAsync(z.first, 0, z.second, st));
         VQ_CUDA(cudaEventRecordWithFlags(e0, st, flags));
         fn<<<ctas, stages == 6 ? batch_threads<6>() : batch_threads<4>(), smem, st>>>(a);
         VQ_LAUNCH_CHECK("batch kernel");
@@ -781,10 +780,6 @@ int batch_run(veloxq_ctx* const* ctxs, int32_t count, int32_t R, const RunParams
             key.push_back(u);
         }
         for (int t = 0; t < 4; ++t) key.push_back(rwork[t].size());
-        for (const auto& z : zero) {
-            key.push_back((uint64_t)(uintptr_t)z.first);
-            key.push_back(z.second);
-        }
         if (!graph->exec || graph->key != key) {
             if (graph->exec) {
                 cudaGraphExecDestroy(graph->exec);

@@ -78,8 +78,10 @@ __global__ void k_best_bits_nr(int64_t n, int32_t R, const float* __restrict__ S
     bits[(int64_t)r * nw + w] = word;
 }
 
-// argmin over replicas (lowest index on ties) -> misc[0]
-__global__ void k_argmin(int32_t R, const int64_t* __restrict__ best, int64_t* misc) {
+// argmin over replicas (lowest index on ties) -> misc[0], its energy ->
+// misc[1]; with x, the winner's vector too (small n: one launch less)
+__global__ void k_argmin(int32_t R, const int64_t* __restrict__ best, int64_t* misc, int64_t n,
+                         const uint32_t* __restrict__ bits, uint8_t* x) {
     __shared__ int64_t sv[1024];
     __shared__ int32_t si[1024];
     int64_t bv = INT64_MAX;
@@ -105,6 +107,10 @@ __global__ void k_argmin(int32_t R, const int64_t* __restrict__ best, int64_t* m
     if (threadIdx.x == 0) {
         misc[0] = si[0];
         misc[1] = sv[0];
+    }
+    if (x) {
+        const uint32_t* w = bits + (int64_t)si[0] * ((n + 31) / 32);
+        for (int64_t i = threadIdx.x; i < n; i += blockDim.x) x[i] = (uint8_t)((w[i >> 5] >> (i & 31)) & 1u);
     }
 }
 
@@ -233,8 +239,9 @@ int launch_best_bits(veloxq_ctx* ctx, int32_t R, Layout layout, const float* S, 
 
 int launch_argmin_unpack(veloxq_ctx* ctx, int32_t R, const int64_t* best, const uint32_t* bits, int64_t* misc,
                          uint8_t* x) {
-    k_argmin<<<1, 1024, 0, ctx->stream>>>(R, best, misc);
-    if (x) k_unpack<<<(unsigned)div_up(ctx->n, 256), 256, 0, ctx->stream>>>(ctx->n, bits, misc, x);
+    const bool small = ctx->n <= 16384;
+    k_argmin<<<1, 1024, 0, ctx->stream>>>(R, best, misc, ctx->n, bits, small ? x : nullptr);
+    if (x && !small) k_unpack<<<(unsigned)div_up(ctx->n, 256), 256, 0, ctx->stream>>>(ctx->n, bits, misc, x);
     VQ_LAUNCH_CHECK("argmin");
     return VELOXQ_OK;
 }

@@ -138,7 +138,14 @@ struct veloxq_ctx {
     vq::DevBuf dfix;              // int64  [n] round((Q_ii + c_i) 2^S)
 
     // ---- scratch reused across calls ----
-    vq::DevBuf s_a, s_b, y, f, ework, best_e, best_bits, flags, a_table, xout, misc;
+    vq::DevBuf s_a, s_b, y, f, ework, best_bits, flags, a_table;
+    std::vector<float> a_host;    // the a(t) values a_table holds (empty: none)
+    // results of a solve, brought to the host in one copy: winner's replica and
+    // energy, each replica's best energy, the winner's vector
+    vq::DevBuf res;
+    int64_t* res_win() const { return res.as<int64_t>(); }                                        // [2]
+    int64_t* res_best() const { return res.as<int64_t>() + 2; }                                   // [R]
+    uint8_t* res_x(int64_t R) const { return reinterpret_cast<uint8_t*>(res.as<int64_t>() + 2 + R); }   // [n]
     vq::DevBuf sop_a, sop_b;      // tensor-core operand copies of S (ping-pong)
     vq::DevBuf dpart;             // float [ksplit][R][n] split-k partial fields of the FP32 dense step
     // FP32 field on the tensor cores (vq_tc32.cu)
@@ -233,9 +240,9 @@ struct BatchGraph {
 };
 // stages: pipeline depth (4 or 6); split: replica groups per instance, each a
 // work item of R / split replicas (a multiple of 16); graph (or null): run the
-// device part as a captured graph kept there
+// device part as a captured graph kept there; d_x: the winners' vectors, one after the other
 int batch_run(veloxq_ctx* const* ctxs, int32_t count, int32_t R, const RunParams& p, uint64_t seed, cudaStream_t st,
-              int stages, int split, DevBuf& work, int64_t* d_best_all, int* d_err, float* ms_main,
+              int stages, int split, DevBuf& work, int64_t* d_best_all, uint8_t* d_x, int* d_err, float* ms_main,
               int64_t* launches = nullptr, BatchGraph* graph = nullptr);
 
 // adjoint of the step (vq_adjoint.cu); the timing covers the whole gradient
