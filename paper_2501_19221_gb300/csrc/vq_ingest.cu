@@ -411,6 +411,12 @@ __device__ __forceinline__ void lz_block_finish(float v, LzScal sc, double* out)
         *sc.count = 0u;
     }
 }
+// The passes are launched dependently: nothing the previous one wrote is read
+// before this wait.
+__device__ __forceinline__ void lz_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 // w_0 = the fixed start vector; |w_0|^2
 __global__ void __launch_bounds__(kPiBlock) k_lz_start(int64_t n, float* __restrict__ w, LzScal sc) {
     float sq = 0.0f;
@@ -426,15 +432,15 @@ __global__ void __launch_bounds__(kPiBlock) k_lz_start(int64_t n, float* __restr
 // (still in L2) come first.
 __global__ void __launch_bounds__(kPiBlock) k_lz_spmv(int64_t n, const int64_t* __restrict__ rp,
                                                      const int32_t* __restrict__ col, const float* __restrict__ wf,
-                                                     const float* __restrict__ wj, float* __restrict__ u, LzScal sc,
-                                                     int j) {
-    const float inv = inv_norm(sc.nrm2[j]);
+                                                     const float* wj, float* u, LzScal sc, int j) {
+    lz_wait();
+    const float inv = inv_norm(*(volatile double*)(sc.nrm2 + j));
     const bool rev = j & 1;
     float dot = 0.0f;
     for (int64_t k = (int64_t)blockIdx.x * kPiBlock + threadIdx.x; k < n; k += (int64_t)gridDim.x * kPiBlock) {
         const int64_t i = rev ? n - 1 - k : k;
         float a = 0.0f;
-        for (int64_t p = rp[i]; p < rp[i + 1]; ++p) a = fmaf(wf[p], wj[col[p]], a);
+        for (int64_t p = rp[i]; p < rp[i + 1]; ++p) a = fmaf(wf[p], __ldca(wj + col[p]), a);
         a *= inv;
         u[i] = a;
         dot = fmaf(a, wj[i] * inv, dot);
@@ -442,10 +448,13 @@ __global__ void __launch_bounds__(kPiBlock) k_lz_spmv(int64_t n, const int64_t* 
     lz_block_finish(dot, sc, sc.alpha + j);
 }
 // The same for a dense Qoff: one warp per row, 16-byte loads when n % 4 == 0.
+// KEEP: Qoff fits in L2 and is read with the normal policy, so that every pass
+// after the first reads it from there; else evict-first.
+template <bool KEEP>
 __global__ void __launch_bounds__(kPiBlock) k_lz_gemv(int64_t n, const float* __restrict__ q,
-                                                     const float* __restrict__ wj, float* __restrict__ u, LzScal sc,
-                                                     int j) {
-    const float inv = inv_norm(sc.nrm2[j]);
+                                                     const float* wj, float* u, LzScal sc, int j) {
+    lz_wait();
+    const float inv = inv_norm(*(volatile double*)(sc.nrm2 + j));
     const bool rev = j & 1;
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = (int64_t)gridDim.x * (kPiBlock / 32);
@@ -464,8 +473,8 @@ __global__ void __launch_bounds__(kPiBlock) k_lz_gemv(int64_t n, const float* __
                 float4 x[8], y[8];
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
-                    x[u] = __ldcs(r4 + c + u * 32);
-                    y[u] = v4[c + u * 32];
+                    x[u] = KEEP ? __ldca(r4 + c + u * 32) : __ldcs(r4 + c + u * 32);
+                    y[u] = __ldca(v4 + c + u * 32);
                 }
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
@@ -476,14 +485,14 @@ __global__ void __launch_bounds__(kPiBlock) k_lz_gemv(int64_t n, const float* __
                 }
             }
             for (; c < n4; c += 32) {
-                const float4 x = __ldcs(r4 + c), y = v4[c];
+                const float4 x = KEEP ? __ldca(r4 + c) : __ldcs(r4 + c), y = __ldca(v4 + c);
                 a = fmaf(x.x, y.x, a);
                 a = fmaf(x.y, y.y, a);
                 a = fmaf(x.z, y.z, a);
                 a = fmaf(x.w, y.w, a);
             }
         } else {
-            for (int64_t c = lane; c < n; c += 32) a = fmaf(row[c], wj[c], a);
+            for (int64_t c = lane; c < n; c += 32) a = fmaf(row[c], __ldca(wj + c), a);
         }
         a = warp_sum_to_lane0(a);
         if (lane == 0) {
@@ -496,11 +505,13 @@ __global__ void __launch_bounds__(kPiBlock) k_lz_gemv(int64_t n, const float* __
 }
 // w_{j+1} = u - alpha_j v_j - beta_j v_{j-1} in place of u, and |w_{j+1}|^2
 // (beta_j = |w_j|, v_j = w_j / |w_j|).
-__global__ void __launch_bounds__(kPiBlock) k_lz_update(int64_t n, float* __restrict__ u, const float* __restrict__ wj,
-                                                       const float* __restrict__ wjm1, LzScal sc, int j) {
-    const double nj = sc.nrm2[j];
-    const float c1 = (float)(sc.alpha[j] * (nj > 0.0 ? 1.0 / sqrt(nj) : 0.0));
-    const float c2 = (j > 0 && sc.nrm2[j - 1] > 0.0) ? (float)sqrt(nj / sc.nrm2[j - 1]) : 0.0f;
+__global__ void __launch_bounds__(kPiBlock) k_lz_update(int64_t n, float* u, const float* wj, const float* wjm1,
+                                                       LzScal sc, int j) {
+    lz_wait();
+    const volatile double *nrm2 = sc.nrm2, *alpha = sc.alpha;
+    const double nj = nrm2[j], nm = j > 0 ? nrm2[j - 1] : 0.0;
+    const float c1 = (float)(alpha[j] * (nj > 0.0 ? 1.0 / sqrt(nj) : 0.0));
+    const float c2 = nm > 0.0 ? (float)sqrt(nj / nm) : 0.0f;
     float sq = 0.0f;
     for (int64_t i = (int64_t)blockIdx.x * kPiBlock + threadIdx.x; i < n; i += (int64_t)gridDim.x * kPiBlock) {
         float w = fmaf(-c1, wj[i], u[i]);
@@ -1023,15 +1034,22 @@ int power_iteration(veloxq_ctx* ctx, int iters, double* rho) {
     sc.count = reinterpret_cast<unsigned*>(sc.nrm2 + kLzSteps + 2);
     VQ_CUDA(cudaMemsetAsync(sc.count, 0, sizeof(unsigned), st));
     k_lz_start<<<grid, kPiBlock, 0, st>>>(n, wv[0], sc);
+    // The passes are launched dependently: 64 short kernels, each waiting for
+    // the one before it inside. Qoff stays in L2 between passes up to 96 MB
+    // (n = 4896).
+    const bool keep = ctx->dense && (double)n * (double)n * 4.0 <= 96e6;
     for (int j = 0; j < m; ++j) {
         float* wj = wv[j % 3];
         float* u = wv[(j + 1) % 3];
         if (ctx->dense)
-            k_lz_gemv<<<grid, kPiBlock, 0, st>>>(n, ctx->qoff32.as<float>(), wj, u, sc, j);
+            VQ_CUDA(launch_dependent(true, keep ? k_lz_gemv<true> : k_lz_gemv<false>, dim3(grid), dim3(kPiBlock), 0, st, n,
+                                     ctx->qoff32.as<float>(), wj, u, sc, j));
         else
-            k_lz_spmv<<<grid, kPiBlock, 0, st>>>(n, ctx->rowptr.as<int64_t>(), ctx->col.as<int32_t>(),
-                                                 ctx->wf.as<float>(), wj, u, sc, j);
-        if (j + 1 < m) k_lz_update<<<ugrid, kPiBlock, 0, st>>>(n, u, wj, wv[(j + 2) % 3], sc, j);
+            VQ_CUDA(launch_dependent(true, k_lz_spmv, dim3(grid), dim3(kPiBlock), 0, st, n, ctx->rowptr.as<int64_t>(),
+                                     ctx->col.as<int32_t>(), ctx->wf.as<float>(), wj, u, sc, j));
+        if (j + 1 < m)
+            VQ_CUDA(launch_dependent(true, k_lz_update, dim3(ugrid), dim3(kPiBlock), 0, st, n, u, wj, wv[(j + 2) % 3], sc,
+                                     j));
     }
     VQ_LAUNCH_CHECK("Lanczos");
     std::vector<double> al((size_t)m), n2((size_t)m);

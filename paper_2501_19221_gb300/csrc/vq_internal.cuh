@@ -186,6 +186,24 @@ int launch_best_bits(veloxq_ctx* ctx, int32_t R, Layout layout, const float* S, 
 int launch_argmin_unpack(veloxq_ctx* ctx, int32_t R, const int64_t* best, const uint32_t* bits,
                          int64_t* misc, uint8_t* x);
 
+// Launch; dependent: by programmatic dependent launch, so that the kernel may
+// become resident while the previous one on the stream drains and waits for
+// it itself (griddepcontrol.wait before it reads anything that one wrote).
+template <typename... P, typename... A>
+cudaError_t launch_dependent(bool dependent, void (*fn)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = dependent ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, fn, static_cast<P>(args)...);
+}
+
 // The integrator of a step (veloxq_method) and PA's momentum.
 struct Rule {
     int method = 0;
