@@ -557,7 +557,7 @@ def roofline(B, w, runner, path, main_ms, main_launches):
     # pointers are read only when rows differ in length (rows of equal length start at i * degree)
     per_nnz = 5 if runner.int8_couplings else 8
     hbm_bytes = 16 * n * R + per_nnz * runner.nnz_field + (0 if runner.regular else 8 * (n + 1))
-    per = main_ms / max(1, main_launches)
+    per = main_ms / K
     ach = hbm_bytes / (per / 1e3) / 1e9
     return {"kernel": "k_stream_step", "bound": "hbm", "achieved": ach, "peak": peaks["hbm_gbs"], "unit": "GB/s",
             "frac": ach / peaks["hbm_gbs"], "traffic": None, "peak_source": f"{src} hbm_gbs",

@@ -170,7 +170,9 @@ typedef struct {
                                VELOXQ_STREAM_FORM="gather chunk", chunk in replicas as in stream_chunk,
                                EINVAL if it does not fit); else 0 */
     int32_t stream_chunk;   /* streaming path: replicas per chunk of the step's thread order (every row of
-                               one chunk before the next; 0: all replicas at once); else 0 */
+                               one chunk before the next; 0: all replicas at once), or per window where the
+                               steps between two readouts run for one window of replicas after the other
+                               (main_launches then counts one per window and step); else 0 */
     int32_t batch_stages;   /* one-launch veloxq_solve_batch: pipeline stages of the autotuned form; else 0 */
     int32_t batch_group;    /* one-launch veloxq_solve_batch: replicas per work item (an instance's
                                replicas in groups of this size, each on its own CTA); else 0 */

@@ -429,6 +429,7 @@ bool is_readout(const RunParams& p, int k) {
 // readout energies in the tensor-core form (sized before the capture).
 int enqueue_loop(veloxq_ctx* ctx, veloxq_path path, int32_t R, const RunParams& p, int nparts, const TcRun* tc,
                  T32Run* t32, bool tc_energy, cudaEvent_t ev_steps) {
+    const bool window = std::getenv("VELOXQ_STREAM_FORM") == nullptr;   // a form fixed by the caller runs as given
     const Layout lay = path == VELOXQ_PATH_DENSE ? LAYOUT_RN : LAYOUT_NR;
     float* cur = ctx->s_a.as<float>();
     float* nxt = ctx->s_b.as<float>();
@@ -458,7 +459,21 @@ int enqueue_loop(veloxq_ctx* ctx, veloxq_path path, int32_t R, const RunParams& 
         } else if (path == VELOXQ_PATH_DENSE) {
             VQ_TRY(dense_step(ctx, R, cur, nxt, Y, at, k, p.dt, p.a0, p.c0, nullptr, rule_of(p)));
         } else {
-            VQ_TRY(stream_step(ctx, R, cur, nxt, Y, at, k, p.dt, p.a0, p.c0, nullptr, rule_of(p)));
+            int k1 = k;
+            while (!is_readout(p, k1)) ++k1;
+            const int32_t win = window ? stream_window(ctx, R, k1 + 1 - k) : 0;
+            if (win) {
+                // the steps up to the readout, one window of replicas after the other
+                for (int32_t r = 0; r < R; r += win) {
+                    float *c = cur, *x = nxt;
+                    for (int q = k; q <= k1; ++q, std::swap(c, x))
+                        VQ_TRY(stream_step(ctx, R, c, x, Y, at, q, p.dt, p.a0, p.c0, nullptr, rule_of(p), r, win));
+                }
+                if (!((k1 + 1 - k) & 1)) std::swap(cur, nxt);   // undone by the exchange below: an even run ends in cur
+                k = k1;
+            } else {
+                VQ_TRY(stream_step(ctx, R, cur, nxt, Y, at, k, p.dt, p.a0, p.c0, nullptr, rule_of(p)));
+            }
         }
         if (!tc && !t32) std::swap(cur, nxt);
         // an event node of the graph (a plain record during capture would only order streams)
@@ -762,6 +777,16 @@ int veloxq_solve(veloxq_ctx* ctx, int32_t replicas, int32_t steps, const veloxq_
         VQ_CUDA(cudaEventRecord(ex->t3, ctx->stream));
         launches = 1 + (use_tc || use_t32 ? 1 : 0) + ex->graph_launches;   // init (+ operand) kernels + graph nodes
         main_launches = steps;
+        if (path == VELOXQ_PATH_STREAM && !std::getenv("VELOXQ_STREAM_FORM")) {
+            main_launches = 0;
+            for (int k = 0, from = 0; k < steps; ++k)
+                if (is_readout(p, k)) {
+                    const int32_t win = stream_window(ctx, replicas, k + 1 - from);
+                    main_launches += (k + 1 - from) * (win ? replicas / win : 1);
+                    window = std::max(window, win);
+                    from = k + 1;
+                }
+        }
         if (use_t32) {
             main_launches = 0;
             for (int k = 0, from = 0; k < steps; ++k)
@@ -799,7 +824,7 @@ int veloxq_solve(veloxq_ctx* ctx, int32_t replicas, int32_t steps, const veloxq_
         ex->timing.main_launches = main_launches;
         const bool streamed = path == VELOXQ_PATH_STREAM;
         ex->timing.stream_gather = streamed ? ctx->stream_unroll : 0;
-        ex->timing.stream_chunk = streamed ? ctx->stream_cvec * vec_width(replicas) : 0;
+        ex->timing.stream_chunk = streamed ? (window ? window : ctx->stream_cvec * vec_width(replicas)) : 0;
         ex->timing.batch_stages = 0;
         ex->timing.batch_group = 0;
         ex->timed = true;

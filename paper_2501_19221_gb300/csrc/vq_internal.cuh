@@ -213,7 +213,9 @@ inline Rule rule_of(const RunParams& p) { return Rule{p.method, p.alpha}; }
 
 // sparse streaming kernels (vq_stream.cu)
 int stream_step(veloxq_ctx* ctx, int32_t R, const float* S_cur, float* S_nxt, float* Y,
-                const float* a_table, int k, float dt, float a0, float c0, float* F_out, const Rule& rule = Rule());
+                const float* a_table, int k, float dt, float a0, float c0, float* F_out, const Rule& rule = Rule(),
+                int32_t r0 = 0, int32_t rn = 0);   // rn > 0: replicas [r0, r0 + rn) only
+int32_t stream_window(const veloxq_ctx* ctx, int32_t R, int steps);
 int stream_energy(veloxq_ctx* ctx, int32_t R, const float* S, int64_t* parts, int* nparts);
 int stream_field(veloxq_ctx* ctx, int32_t R, const float* S, float* F);
 int stream_step_y(veloxq_ctx* ctx, int32_t R, const float* S_cur, float* S_nxt, const float* Y_in, float* Y_out,

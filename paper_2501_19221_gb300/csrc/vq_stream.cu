@@ -179,10 +179,17 @@ __global__ void __launch_bounds__(256) k_sparse_energy_x(int64_t n, int64_t B, c
 
 template <bool FIELD_ONLY, bool SIGN>
 int launch_step(veloxq_ctx* ctx, int32_t R, const float* S_cur, float* S_nxt, const float* Y_in, float* Y_out,
-                const float* a_table, int k, float dt, float a0, float c0, float* F_out, const Rule& rule) {
+                const float* a_table, int k, float dt, float a0, float c0, float* F_out, const Rule& rule,
+                int32_t r0 = 0, int32_t rn = 0) {
     const int V = vec_width(R);
-    const int32_t nvec = R / V;
-    const int32_t cvec = (ctx->stream_cvec > 0 && nvec % ctx->stream_cvec == 0) ? ctx->stream_cvec : nvec;
+    const int32_t nvec = (rn ? rn : R) / V;
+    // a window of replicas: the same rows, from its first replica on
+    S_cur += r0;
+    if (S_nxt) S_nxt += r0;
+    if (Y_in) Y_in += r0;
+    if (Y_out) Y_out += r0;
+    if (F_out) F_out += r0;
+    const int32_t cvec = (!rn && ctx->stream_cvec > 0 && nvec % ctx->stream_cvec == 0) ? ctx->stream_cvec : nvec;
     const int64_t total = ctx->n * (int64_t)nvec;
     const unsigned g = (unsigned)div_up(total, 256);
     // Short steps are launched dependently, so that a step's launch and first
@@ -236,10 +243,31 @@ int launch_step(veloxq_ctx* ctx, int32_t R, const float* S_cur, float* S_nxt, co
 int vec_width(int32_t R) { return (R % 4 == 0) ? 4 : (R % 2 == 0) ? 2 : 1; }
 
 int stream_step(veloxq_ctx* ctx, int32_t R, const float* S_cur, float* S_nxt, float* Y, const float* a_table, int k,
-                float dt, float a0, float c0, float* F_out, const Rule& rule) {
+                float dt, float a0, float c0, float* F_out, const Rule& rule, int32_t r0, int32_t rn) {
     if (rule.method == VELOXQ_METHOD_PA)
-        return launch_step<false, true>(ctx, R, S_cur, S_nxt, Y, Y, a_table, k, dt, a0, c0, F_out, rule);
-    return launch_step<false, false>(ctx, R, S_cur, S_nxt, Y, Y, a_table, k, dt, a0, c0, F_out, rule);
+        return launch_step<false, true>(ctx, R, S_cur, S_nxt, Y, Y, a_table, k, dt, a0, c0, F_out, rule, r0, rn);
+    return launch_step<false, false>(ctx, R, S_cur, S_nxt, Y, Y, a_table, k, dt, a0, c0, F_out, rule, r0, rn);
+}
+
+// Replicas per window of a run of steps (0: all at once). Replicas are
+// independent, so the steps between two readouts may run for one window of
+// replicas after the other. When the state of all replicas lies well beyond
+// L2 but a window's two state arrays and momenta stay in it with the
+// couplings, every step after a window's first reads and writes L2 instead
+// of HBM. The widest window of at most 96 MB is taken (L2 holds 126 MB), of at
+// least 32 replicas (one 128-byte line per row) and 2.5 M variable-replicas
+// (shorter steps cost more in launches than they save).
+int32_t stream_window(const veloxq_ctx* ctx, int32_t R, int steps) {
+    const double l2 = 126e6, room = 96e6;
+    const double couplings = (double)ctx->nnz * (ctx->w8.p ? 5.0 : 8.0) + 12.0 * (double)ctx->n;
+    if (steps < 4 || 12.0 * (double)ctx->n * R + couplings <= 1.5 * l2) return 0;
+    for (int32_t parts = 2; R / parts >= 32; ++parts) {
+        const int32_t w = R / parts;
+        if (R % parts != 0 || w % 32 != 0) continue;
+        if (12.0 * (double)ctx->n * w + couplings > room) continue;
+        return (double)ctx->n * w >= 2.5e6 ? w : 0;
+    }
+    return 0;
 }
 
 int stream_step_y(veloxq_ctx* ctx, int32_t R, const float* S_cur, float* S_nxt, const float* Y_in, float* Y_out,
@@ -311,14 +339,15 @@ int stream_autotune(veloxq_ctx* ctx, int32_t R, float* S_a, float* S_b, float* Y
     VQ_TRY(launch_init_state(ctx, R, 1, 0.1f, LAYOUT_NR, S_a, Y));
     const float* at = ctx->a_table.as<float>();
     std::vector<std::pair<int, int32_t>> cands;   // (gather, chunk)
-    for (int32_t cv : chunk_candidates(ctx->n, R))
+    const int32_t win = stream_window(ctx, R, 50);  // runs by windows: their steps are timed, without chunks
+    for (int32_t cv : win ? std::vector<int32_t>{0} : chunk_candidates(ctx->n, R))
         for (int u : {1, 4, 6})
             if (u != 6 || ctx->uniform_deg == 6) cands.emplace_back(u, cv);
     auto timed = [&](int reps, float* ms) -> int {
         VQ_CUDA(cudaEventRecord(e0, ctx->stream));
         for (int k = 0; k < reps; ++k)
             VQ_TRY((launch_step<false, false>(ctx, R, (k & 1) ? S_b : S_a, (k & 1) ? S_a : S_b, Y, Y, at, 0, 0.5f,
-                                              1.0f, 0.1f, nullptr, Rule())));
+                                              1.0f, 0.1f, nullptr, Rule(), 0, win)));
         VQ_CUDA(cudaEventRecord(e1, ctx->stream));
         VQ_CUDA(cudaEventSynchronize(e1));
         VQ_CUDA(cudaEventElapsedTime(ms, e0, e1));
