@@ -2,31 +2,40 @@
 // 5th-generation tensor cores, with the update fused into the epilogue: the
 // form dense contexts run in VELOXQ_PREC_FP32.
 //
-// Every FP32 operand is written as the exact sum of three BF16 terms of 8
-// significant bits each (x = x1 + x2 + x3, by truncation), and the product is
-// the sum of the six term products down to 2^-16 of the leading one,
+// Every FP32 operand is written as the exact sum of three BF16 terms
+// (x = x1 + x2 + x3: 6, 8 and up to 9 significant bits), and the product is the
+// sum of the six term products down to 2^-16 of the leading one,
 //     q s ~ q1 s1 + (q1 s2 + q2 s1) + (q2 s2 + q1 s3 + q3 s1);
-// the three that are left out are below 2^-23 of q s. Products of BF16 terms
-// are exact in FP32. The accumulators in tensor memory are drained after
-// every 32 variables into FP32 registers with rounded additions, the five
-// small term products of a block accumulated before the leading one, so that
-// no long sum runs through the tensor cores' accumulation. For Parallel
-// Annealing the operand is +-1, one exact term, and three products are the
-// whole of q s.
+// the three that are left out are below 2^-22 of q s. For Parallel Annealing
+// the operand is +-1, one exact term, and three products are the whole of q s.
 //
-// Error against FP64 (normwise, N(0, 1/n) couplings): below that of the FP32
-// SGEMM of vq_dense.cu at every size measured, n = 600 to 8192.
+// Accuracy: the products of BF16 terms are exact in FP32, but the tensor
+// cores' accumulation cuts its sums off toward zero, a relative shrinking that
+// adds up over the steps of a run. Three things keep it small: the leading
+// term has 6 bits only, so that a sum of leading products is mostly exact in
+// 24 bits (with 8-bit leading terms the field shrank by 5.8e-8, with 6 bits by
+// 3e-9 at 32 variables); the five small products go to an accumulator of their
+// own (sharing one: 8.3e-8); and both are drained after every 64 or 128
+// variables into FP32 registers with rounded additions. Error against FP64
+// (normwise, N(0, 1/n) couplings, S uniform in [-1, 1]), the FP32 SGEMM of
+// vq_dense.cu -> here: n = 600: 2.2e-7 -> 1.0e-7, 2048: 2.2e-7 -> 1.1e-7,
+// 4096: 5.1e-7 -> 1.2e-7, 8192: 1.6e-6 -> 1.7e-7.
+//
+// Time per step, SGEMM -> here: n = 8192, R = 1024: 4060 -> 580 us (0.74 of
+// the measured BF16 rate at 12 n^2 R FLOP); n = 8192, R = 64: 650 -> 100 us;
+// n = 3000, R = 1000: 690 -> 130 us; n = 1001, R = 100: 41 -> 13 us.
 //
 // CTA pairs (clusters of 2, cta_group::2) compute 256 x 128 tiles (rows x
 // replicas), M = 256 MMAs issued by the even CTA, operands staged by TMA in
-// blocks of 32 variables: the three terms of a CTA's 128 rows (24 KB) and of
-// its 64 replicas (12 KB) in one 3-D copy each, 5 stages. Tiles of 128
+// blocks of 64 variables: the three terms of a CTA's 128 rows (48 KB) and of
+// its 64 replicas (24 KB) in one 3-D copy each, 3 stages (blocks of 32, whose
+// rows are half as long, took 631 instead of 585 us at n = 8192). Tiles of 128
 // replicas rather than 256 keep a thread's part of the drained field in 64
 // registers, and give twice the tiles to spread over the SMs.
 //   * Enough tiles (more than half of the pairs): one launch runs every step
 //     up to a readout, tiles of consecutive steps overlapping as in vq_tc.cu.
-//   * Fewer: the k-loop is split over the idle pairs (at least 4 blocks of 32
-//     variables each), the partial fields go to a workspace, and
+//   * Fewer: the k-loop is split over the idle pairs (at least two blocks each; with one, 14 against 13 us per
+//     step at n = 1001, R = 100), the partial fields go to a workspace, and
 //     k_t32_finish adds them in order, updates, and writes the next operand.
 //     The two launches of a step follow each other by programmatic dependent
 //     launch. The choice depends on n and R alone, so a run gives the same
@@ -274,23 +283,25 @@ __global__ void __launch_bounds__(THREADS, 1) k_t32(const __grid_constant__ CUte
                     tc_fence_after();
                     const uint32_t d = tmem + b * 2 * BN, dx = d + BN;
                     const uint32_t sa = smem_u32(smem + s * STAGE_BYTES), sb = sa + 3 * A_TERM;
-                    // the leading products into one accumulator, the small ones (smallest first) into another
+                    // the leading products into one accumulator, the small ones into another
 #pragma unroll
                     for (int kk = 0; kk < BK / 16; ++kk) {
                         const uint32_t o = kk * 32, acc = (kk != 0 || !first) ? 1u : 0u;
                         const uint64_t a0 = desc128(sa + o), a1 = desc128(sa + A_TERM + o), a2 = desc128(sa + 2 * A_TERM + o);
                         const uint64_t b0 = desc128(sb + o);
-                        mma_pair(dx, a2, b0, acc);
                         if constexpr (NB == 3) {
                             const uint64_t b1 = desc128(sb + B_TERM + o), b2 = desc128(sb + 2 * B_TERM + o);
-                            mma_pair(dx, a0, b2, 1u);
+                            mma_pair(d, a0, b0, acc);
+                            mma_pair(dx, a0, b2, acc);
+                            mma_pair(dx, a0, b1, 1u);
                             mma_pair(dx, a1, b1, 1u);
                             mma_pair(dx, a1, b0, 1u);
-                            mma_pair(dx, a0, b1, 1u);
+                            mma_pair(dx, a2, b0, 1u);
                         } else {
+                            mma_pair(d, a0, b0, acc);
+                            mma_pair(dx, a2, b0, acc);
                             mma_pair(dx, a1, b0, 1u);
                         }
-                        mma_pair(d, a0, b0, acc);
                     }
                     umma_commit_pair(&empty[s]);
                     if (last) {
@@ -412,22 +423,35 @@ __global__ void __launch_bounds__(THREADS, 1) k_t32(const __grid_constant__ CUte
 // step's operand. FIELD: the field alone.
 template <int NB, int FORM>
 __global__ void __launch_bounds__(256) k_t32_finish(const T32Args a) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (a.skip && *a.skip == a.skip_seq) return;
     const int nb = (a.n + 255) / 256;
     const int64_t r = blockIdx.x / nb;
     const int i = (int)(blockIdx.x - r * nb) * 256 + threadIdx.x;
-    if (i >= a.n) return;
     const int64_t p = r * a.n + i, total = (int64_t)a.R * a.n;
+    // This kernel starts when every CTA of the field kernel has passed its own
+    // wait, so the state (written by the previous step's k_t32_finish) may be
+    // read before this one; the partial fields only after it.
     float s = 0.0f, y = 0.0f;
     if constexpr (FORM != FORM_FIELD) {
-        s = a.S_a[p];
-        y = a.Y[p];
+        if (i < a.n) {
+            s = __ldcg(a.S_a + p);
+            y = __ldcg(a.Y + p);
+        }
     }
-    float F = a.part[p];
-#pragma unroll 4
-    for (int z = 1; z < a.ksplit; ++z) F = __fadd_rn(F, a.part[(int64_t)z * total + p]);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (i >= a.n || (a.skip && *a.skip == a.skip_seq)) return;
+    // eight partial fields in flight, added in order
+    float F = 0.0f;
+    for (int z0 = 0; z0 < a.ksplit; z0 += 8) {
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = z0 + u < a.ksplit ? __ldcs(a.part + (int64_t)(z0 + u) * total + p) : 0.0f;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            if (z0 + u == 0) F = v[0];
+            else if (z0 + u < a.ksplit) F = __fadd_rn(F, v[u]);
+        }
+    }
     if (a.F_out) a.F_out[p] = F;
     if constexpr (FORM != FORM_FIELD) {
         const float bi = __ldg(a.bf + i), a_k = __ldg(a.a_table + a.k);
