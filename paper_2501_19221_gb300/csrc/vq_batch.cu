@@ -577,7 +577,13 @@ int batch_run(veloxq_ctx* const* ctxs, int32_t count, int32_t R, const RunParams
               int stages, int split, DevBuf& work, int64_t* d_best_all, uint8_t* d_x, int* d_err, float* ms_main,
               int64_t* launches, BatchGraph* graph) {
     int64_t nl = 0;
-    std::vector<std::pair<void*, size_t>> zero;   // operand buffers whose padding is zeroed
+    // contexts whose operand buffers' padding is zeroed, and the layout they then hold
+    struct Pad {
+        veloxq_ctx* c;
+        size_t bytes;
+        int64_t tag;
+    };
+    std::vector<Pad> zero;
     const int terms = batch_terms(p.prec, p.method);
     if (split < 1 || R % split != 0 || (R / split) % 16 != 0)
         return fail(VELOXQ_EINVAL, "replica groups must hold a multiple of 16 replicas");
@@ -626,9 +632,8 @@ int batch_run(veloxq_ctx* const* ctxs, int32_t count, int32_t R, const RunParams
         // captured part
         const int64_t tag = ((int64_t)R << 16) | ((int64_t)p.prec << 8) | ((int64_t)terms << 4) | 1;
         if (c->sop_tag != tag || c->sop_a.p != pa || c->sop_b.p != pb) {
-            zero.push_back({c->sop_a.p, sopb});
-            zero.push_back({c->sop_b.p, sopb});
-            c->sop_tag = tag;
+            c->sop_tag = 0;
+            zero.push_back({c, sopb, tag});
         }
         BatchInst b{};
         b.n = n;
@@ -742,7 +747,11 @@ int batch_run(veloxq_ctx* const* ctxs, int32_t count, int32_t R, const RunParams
         VQ_CUDA(cudaEventCreate(&e0));
         VQ_CUDA(cudaEventCreate(&e1));
     }
-    for (const auto& z : zero) VQ_CUDA(cudaMemsetAsync(z.first, 0, z.second, st));
+    for (const Pad& z : zero) {
+        VQ_CUDA(cudaMemsetAsync(z.c->sop_a.p, 0, z.bytes, st));
+        VQ_CUDA(cudaMemsetAsync(z.c->sop_b.p, 0, z.bytes, st));
+        z.c->sop_tag = z.tag;
+    }
     // the device part of the solve: the persistent kernel between two timing events, and the final readout (one energy launch per
     // element type of Q in the batch, one finish launch)
     auto enqueue = [&]() -> int {
