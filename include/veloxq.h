@@ -369,7 +369,9 @@ int veloxq_energy_dev_noalloc(veloxq_ctx* ctx, int64_t batch, const uint8_t* X, 
 
 /* ---------------------------------------------------------------------------
  * Pieces of the step, for parity tests and for callers that drive the
- * integration themselves (device pointers, asynchronous).
+ * integration themselves (device pointers, asynchronous). A bounded wait of
+ * the tensor-core kernels that gives up after a call has returned is reported
+ * (ETIMEDOUT) by the next call on the context.
  * ------------------------------------------------------------------------- */
 
 /* Philox initial state S, Y [R][n] for seed and sigma0 (same draw as solve). */

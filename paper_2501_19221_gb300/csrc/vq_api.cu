@@ -171,9 +171,14 @@ struct CtxExtra {
     DevBuf bwork, bbest, berr, bx;
     int tune_stages = 0, tune_split = 0;   // form of the last batched launch headed by this context
     BatchGraph bgraph;                     // its captured device part
+    // the last call that returned before its kernels ended: recorded behind
+    // them, waited for by a call on another stream (they share the scratch)
+    cudaEvent_t aev = nullptr;
+    cudaStream_t astream = nullptr;
+    bool apending = false;
     ~CtxExtra() {
         if (graph) cudaGraphExecDestroy(graph);
-        for (cudaEvent_t e : {ev, t0, t1, t2, t3})
+        for (cudaEvent_t e : {ev, aev, t0, t1, t2, t3})
             if (e) cudaEventDestroy(e);
         if (work) cudaStreamDestroy(work);
     }
@@ -313,9 +318,8 @@ int tc_setup(veloxq_ctx* ctx, int prec, int32_t R, TcRun* t, int method = VELOXQ
     // completion counters of multi-step runs, one per replica column block (sized before any capture)
     VQ_TRY(ctx->tcdone.ensure(sizeof(uint32_t) * (size_t)div_up(R, 64)));
     // the K padding columns [n, n_pad) of both operand buffers must stay zero:
-    // the epilogue never writes them
-    VQ_CUDA(cudaMemsetAsync(ctx->sop_a.p, 0, b, ctx->stream));
-    VQ_CUDA(cudaMemsetAsync(ctx->sop_b.p, 0, b, ctx->stream));
+    // tc_quant_s writes them in the first, the epilogue never writes them
+    if (tc_pad(ctx->n) != ctx->n) VQ_CUDA(cudaMemsetAsync(ctx->sop_b.p, 0, b, ctx->stream));
     ctx->sop_tag = 0;
     t->sop[0] = ctx->sop_a.p;
     t->sop[1] = ctx->sop_b.p;
@@ -408,7 +412,28 @@ int check_device(veloxq_ctx* ctx) {
     if (dev != ctx->device)
         return fail(VELOXQ_EINVAL, "the context was created on device " + std::to_string(ctx->device) +
                                        ", which must be the current device (current: " + std::to_string(dev) + ")");
+    CtxExtra* ex = extra(ctx);
+    if (ex && ex->apending && ex->astream != ctx->stream) {
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        VQ_CUDA(cudaStreamIsCapturing(ctx->stream, &cs));
+        if (cs == cudaStreamCaptureStatusNone) {
+            VQ_CUDA(cudaStreamWaitEvent(ctx->stream, ex->aev, 0));
+            ex->apending = false;
+        }
+    }
     return t32_check(ctx);
+}
+
+// Behind the kernels of a call that returns before they end.
+int returns_early(veloxq_ctx* ctx) {
+    CtxExtra* ex = extra(ctx);
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    VQ_CUDA(cudaStreamIsCapturing(ctx->stream, &cs));
+    if (!ex || cs != cudaStreamCaptureStatusNone) return VELOXQ_OK;
+    VQ_CUDA(cudaEventRecord(ex->aev, ctx->stream));
+    ex->astream = ctx->stream;
+    ex->apending = true;
+    return VELOXQ_OK;
 }
 
 int check_err_word(veloxq_ctx* ctx) {
@@ -543,6 +568,7 @@ static int new_ctx(veloxq_ctx** out, int64_t n, void* stream, veloxq_ctx** made)
     auto ex = std::make_unique<CtxExtra>();
     e = cudaStreamCreateWithFlags(&ex->work, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ex->ev, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ex->aev, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreate(&ex->t0);
     if (e == cudaSuccess) e = cudaEventCreate(&ex->t1);
     if (e == cudaSuccess) e = cudaEventCreate(&ex->t2);
@@ -1057,14 +1083,16 @@ int veloxq_field_dev(veloxq_ctx* ctx, int32_t R, veloxq_prec prec, const float* 
             T32Run t;
             VQ_TRY(t32_split(ctx, R, S, Rule(), true, &t));
             VQ_TRY(t32_run(ctx, R, &t, nullptr, nullptr, nullptr, nullptr, 0, 1, 0.f, 0.f, 0.f, F, Rule(), true, true));
-            return dense_field(ctx, R, S, F, ctx->t32w.as<uint32_t>() + 1, t.seq);
+            VQ_TRY(dense_field(ctx, R, S, F, ctx->t32w.as<uint32_t>() + 1, t.seq));
+            return returns_early(ctx);
         }
         TcRun tc;
         VQ_TRY(tc_setup(ctx, prec, R, &tc));
-        VQ_CUDA(cudaMemsetAsync(ctx->errw.p, 0, sizeof(int), ctx->stream));
+        VQ_TRY(async_words(ctx));
         VQ_TRY(tc_quant_s(ctx, prec, R, S, tc.sop[0]));
-        VQ_TRY(tc_field(ctx, prec, R, tc.mq, tc.ms[0], tc.lo(0), F, ctx->errw.as<int>()));
-        return check_err_word(ctx);
+        VQ_TRY(tc_field(ctx, prec, R, tc.mq, tc.ms[0], tc.lo(0), F, ctx->t32w.as<int>(),
+                        static_cast<int*>(ctx->t32h.dev)));
+        return returns_early(ctx);
     }
     if (prec != VELOXQ_PREC_FP32) return fail(VELOXQ_EUNSUPPORTED, "sparse contexts run the field in FP32 (or exact int8)");
     const int64_t nR = ctx->n * (int64_t)R;
@@ -1115,19 +1143,20 @@ int veloxq_steps_dev(veloxq_ctx* ctx, int32_t R, int32_t k_begin, int32_t k_coun
         if (t32) {
             VQ_TRY(t32_run(ctx, R, &t32r, &cur, &nxt, Y, at, k_begin, k_end, p.dt, p.a0, p.c0, F_last, rule_of(p), false,
                            false));
-            return give_back();
+            VQ_TRY(give_back());
+            return returns_early(ctx);
         }
         if (p.prec != VELOXQ_PREC_FP32) {
             TcRun tc;
             VQ_TRY(tc_setup(ctx, p.prec, R, &tc, p.method));
-            VQ_CUDA(cudaMemsetAsync(ctx->errw.p, 0, sizeof(int), ctx->stream));
+            VQ_TRY(async_words(ctx));
             VQ_TRY(tc_quant_s(ctx, p.prec, R, cur, tc.sop[0], rule_of(p)));
             // the whole range in one launch (the solve's form)
             VQ_TRY(tc_run(ctx, p.prec, R, tc.mq, tc.ms, tc.lo(), 0, cur, nxt, Y, tc.sop, at, k_begin, k_end, p.dt,
-                          p.a0, p.c0, F_last, ctx->errw.as<int>(), rule_of(p)));
+                          p.a0, p.c0, F_last, ctx->t32w.as<int>(), rule_of(p), static_cast<int*>(ctx->t32h.dev)));
             if (k_count & 1) std::swap(cur, nxt);
             VQ_TRY(give_back());
-            return check_err_word(ctx);
+            return returns_early(ctx);
         }
         for (int k = k_begin; k < k_end; ++k) {
             VQ_TRY(dense_step(ctx, R, cur, nxt, Y, at, k, p.dt, p.a0, p.c0, k == k_end - 1 ? F_last : nullptr,

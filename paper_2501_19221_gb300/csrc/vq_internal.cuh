@@ -152,7 +152,9 @@ struct veloxq_ctx {
     int q3_state = 0;             // term planes of Qoff: 0 not built yet, 1 built, -1 not used
     vq::DevBuf q3;                // bf16 [3][n][n_pad] Qoff in three exact terms
     vq::DevBuf s3[2];             // bf16 [3][R][n_pad] operand terms of S (ping-pong)
-    vq::DevBuf t32w;              // [0] error word of its waits, [1] sequence number of the last operand out of range
+    // words of the calls that return before their kernels end: [0] error word of the bounded waits, [1] sequence
+    // number of the last FP32 operand out of range
+    vq::DevBuf t32w;
     vq::PinnedWords t32h;         // the same two words where the host can see them without a copy
     uint32_t t32_seq = 0;
     vq::DevBuf errw;              // device error word of bounded waits
@@ -293,10 +295,10 @@ int tc_wait_selftest(long long budget, int* code_out);   // the bounded wait run
 int tc_run(veloxq_ctx* ctx, int prec, int32_t R, const CUtensorMap& mq, const CUtensorMap* ms,
            const CUtensorMap* ms_lo, int cur, const float* S_a, float* S_b, float* Y, void* const* sop,
            const float* a_table, int k_begin, int k_end, float dt, float a0, float c0, float* F_out, int* err,
-           const Rule& rule = Rule());
+           const Rule& rule = Rule(), int* err_host = nullptr);
 // The field alone, F = Qoff S, of the operand behind ms (and ms_lo).
 int tc_field(veloxq_ctx* ctx, int prec, int32_t R, const CUtensorMap& mq, const CUtensorMap& ms,
-             const CUtensorMap* ms_lo, float* F_out, int* err);
+             const CUtensorMap* ms_lo, float* F_out, int* err, int* err_host = nullptr);
 int tc_tile(const veloxq_ctx* ctx, int prec, int terms, int32_t R);   // replicas per tile: 256, 128 or 64
 int tc_operand_map(veloxq_ctx* ctx, CUtensorMap* m, void* base, int prec, int64_t rows, int64_t n_pad, bool a_operand);
 int launch_sum_parts(veloxq_ctx* ctx, int64_t B, int nparts, const int64_t* parts, double* E, int64_t* E_int);
@@ -307,6 +309,7 @@ struct T32Run {
     int terms = 3;        // BF16 terms of the operand
     uint32_t seq = 0;     // sequence number of its range check (0: not checked)
 };
+int async_words(veloxq_ctx* ctx);   // allocates and zeroes t32w and t32h (once)
 int t32_prepare(veloxq_ctx* ctx, int32_t R, bool* ready);
 int t32_split(veloxq_ctx* ctx, int32_t R, const float* S, const Rule& rule, bool check, T32Run* t);
 bool t32_bad(const veloxq_ctx* ctx, const T32Run& t);

@@ -121,6 +121,7 @@ struct TcArgs {
     const float* a_table;
     float* F_out;            // [R][n] field of the last step, or null
     int* err;
+    int* err_host;           // the same word in mapped host memory (calls that return before the kernel ends), or null
     float alpha;             // PA momentum
     int64_t plane;           // elements from the hi plane of an operand buffer to its lo plane (two S terms)
     uint32_t* done;          // [NT] epilogue warps finished per replica column block (zeroed per launch)
@@ -414,6 +415,10 @@ __global__ void __launch_bounds__(320, 1) k_tc_step(const __grid_constant__ CUte
     cluster_sync();
     tc_fence_after();
     if (warp == 1) tmem_dealloc(tmem, 2 * BN);
+    if (threadIdx.x == 0 && a.err_host) {
+        const int e = *(volatile int*)a.err;
+        if (e) atomicOr_system(a.err_host, e);
+    }
 }
 
 // The bounded wait of the kernels above on a barrier that nothing arrives on:
@@ -693,7 +698,7 @@ int tc_column_group(int prec, int terms) {
 int tc_run(veloxq_ctx* ctx, int prec, int32_t R, const CUtensorMap& mq, const CUtensorMap* ms,
            const CUtensorMap* ms_lo, int cur, const float* S_a, float* S_b, float* Y, void* const* sop,
            const float* a_table, int k_begin, int k_end, float dt, float a0, float c0, float* F_out, int* err,
-           const Rule& rule) {
+           const Rule& rule, int* err_host) {
     const bool field_only = S_b == nullptr;
     if (k_end <= k_begin) return VELOXQ_OK;
     if (field_only && k_end != k_begin + 1) return fail(VELOXQ_EINVAL, "the field alone is one step");
@@ -750,6 +755,7 @@ int tc_run(veloxq_ctx* ctx, int prec, int32_t R, const CUtensorMap& mq, const CU
         a.a_table = a_table;
         a.F_out = k1 == k_end ? F_out : nullptr;
         a.err = err;
+        a.err_host = err_host;
         a.alpha = rule.alpha;
         a.plane = (int64_t)R * a.n_pad;
         a.done = nullptr;
@@ -770,12 +776,12 @@ int tc_run(veloxq_ctx* ctx, int prec, int32_t R, const CUtensorMap& mq, const CU
 
 // The field alone, F = Qoff S, from the operand behind ms (and ms_lo).
 int tc_field(veloxq_ctx* ctx, int prec, int32_t R, const CUtensorMap& mq, const CUtensorMap& ms,
-             const CUtensorMap* ms_lo, float* F_out, int* err) {
+             const CUtensorMap* ms_lo, float* F_out, int* err, int* err_host) {
     const CUtensorMap mss[2] = {ms, ms};
     CUtensorMap lo[2];
     if (ms_lo) lo[0] = lo[1] = *ms_lo;
     return tc_run(ctx, prec, R, mq, mss, ms_lo ? lo : nullptr, 0, nullptr, nullptr, nullptr, nullptr, nullptr, 0, 1,
-                  0.f, 0.f, 0.f, F_out, err, Rule());
+                  0.f, 0.f, 0.f, F_out, err, Rule(), err_host);
 }
 
 }  // namespace vq

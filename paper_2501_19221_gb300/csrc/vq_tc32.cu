@@ -639,6 +639,14 @@ int launch_finish(veloxq_ctx* ctx, FinishKernel fn, const T32Args& a) {
 
 }  // namespace
 
+int async_words(veloxq_ctx* ctx) {
+    if (ctx->t32h.p && ctx->t32w.p) return VELOXQ_OK;
+    if (!ctx->t32h.p) VQ_TRY(ctx->t32h.make());
+    VQ_TRY(ctx->t32w.ensure(sizeof(int) * 8));
+    VQ_CUDA(cudaMemsetAsync(ctx->t32w.p, 0, sizeof(int) * 8, ctx->stream));
+    return VELOXQ_OK;
+}
+
 // Prepares the form for R replicas: the term planes of Qoff (once per
 // context), operand and counter buffers. *ready = false (and no error) where
 // the SGEMM has to serve: small n, values whose terms leave BF16's range, or
@@ -671,8 +679,7 @@ int t32_prepare(veloxq_ctx* ctx, int32_t R, bool* ready) {
             VQ_CUDA(cudaMemGetInfo(&free_b, &total_b));
             if (sizeof(__nv_bfloat16) * 3 * (size_t)n * (size_t)np + 2 * ob + pb > free_b / 2) return VELOXQ_OK;
             room(ctx->q3, sizeof(__nv_bfloat16) * 3 * (size_t)n * (size_t)np);
-            room(ctx->t32w, sizeof(int) * 8);
-            if (st == VELOXQ_OK && !ctx->t32h.p && ctx->t32h.make() != VELOXQ_OK) st = VELOXQ_ENOMEM;
+            if (st == VELOXQ_OK) st = async_words(ctx);
         }
         room(ctx->s3[0], ob);
         if (fused) room(ctx->s3[1], ob);
@@ -685,7 +692,6 @@ int t32_prepare(veloxq_ctx* ctx, int32_t R, bool* ready) {
         }
         VQ_TRY(st);
         if (ctx->q3_state == 0) {
-            VQ_CUDA(cudaMemsetAsync(ctx->t32w.p, 0, sizeof(int) * 8, ctx->stream));
             int* bad = ctx->t32w.as<int>() + 2;
             k_t32_split_q<<<(unsigned)n, 256, 0, ctx->stream>>>(n, np, ctx->qoff32.as<float>(),
                                                                 ctx->q3.as<__nv_bfloat16>(), bad);
