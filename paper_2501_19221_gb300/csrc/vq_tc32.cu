@@ -786,7 +786,8 @@ int t32_run(veloxq_ctx* ctx, int32_t R, T32Run* t, float** cur, float** nxt, flo
     // Tensor-core accumulation cuts its sums off toward zero, so F shrinks by a part that grows with the variables
     // between two drains: 3e-9 at 32, 7e-9 at 64, 1.8e-8 at 128. It is kept below about 3 % of the error the FP32
     // SGEMM has at that size (2e-7 up to n = 2048, 5e-7 at 4096, 1.6e-6 at 8192).
-    a.drain = n < 2560 ? 1 : 2;
+    // (Parallel Annealing's products with +-1 have 6 and 8 bits and lose nothing at 256.)
+    a.drain = terms == 1 ? 4 : n < 2560 ? 1 : 2;
     a.err = ctx->t32w.as<int>();
     a.err_host = static_cast<int*>(ctx->t32h.dev);
     a.skip = guard ? ctx->t32w.as<uint32_t>() + 1 : nullptr;
