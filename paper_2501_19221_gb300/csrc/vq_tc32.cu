@@ -58,12 +58,14 @@ namespace {
 
 using namespace tc;
 
-constexpr int BM = 128, BN = 128, BNH = BN / 2;   // rows per CTA; replicas per pair and per CTA
+constexpr int BM = 128;                           // rows per CTA (2 BM per pair)
+constexpr int BN_WIDE = 128, BN_NARROW = 64;      // replicas per pair (half of them staged per CTA)
 constexpr int BK = 64, BKB = 2 * BK;              // variables per block: 128-byte rows
-constexpr uint32_t A_TERM = BM * BKB, B_TERM = BNH * BKB;
-template <int NB> constexpr uint32_t stage_bytes() { return 3 * A_TERM + NB * B_TERM; }
+constexpr uint32_t A_TERM = BM * BKB;
+template <int BN> constexpr uint32_t b_term() { return (BN / 2) * BKB; }
+template <int NB, int BN> constexpr uint32_t stage_bytes() { return 3 * A_TERM + NB * b_term<BN>(); }
 constexpr int STAGES = 3;
-constexpr size_t T32_SMEM = (size_t)STAGES * stage_bytes<3>() + 1024 /*align*/ + 256 /*barriers, slot*/;
+constexpr size_t T32_SMEM = (size_t)STAGES * stage_bytes<3, BN_WIDE>() + 1024 /*align*/ + 256 /*barriers, slot*/;
 constexpr int EPI_WARPS = 8;
 constexpr int THREADS = 32 * (2 + EPI_WARPS);
 constexpr int MIN_BLOCKS = 2;                     // k-blocks per split at least
@@ -110,13 +112,13 @@ __device__ __forceinline__ uint64_t desc128(uint32_t addr) {
            (uint64_t)2 << 61;
 }
 // FP32 accumulator, BF16 operands, K-major, N = BN, M = 2 BM
-constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
+template <int BN> constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
                            ((uint32_t)((2 * BM) >> 4) << 24);
-__device__ __forceinline__ void mma_pair(uint32_t d, uint64_t a, uint64_t b, uint32_t accum) {
+template <int BN> __device__ __forceinline__ void mma_pair(uint32_t d, uint64_t a, uint64_t b, uint32_t accum) {
     asm volatile(
         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}\n"
-        ::"r"(d), "l"(a), "l"(b), "r"(IDESC), "r"(accum)
+        ::"r"(d), "l"(a), "l"(b), "r"(IDESC<BN>), "r"(accum)
         : "memory");
 }
 // box of {64 variables, rows, terms} into this CTA's shared memory
@@ -184,11 +186,13 @@ enum { FORM_BSB = 0, FORM_ASB = 1, FORM_PA = 2, FORM_FIELD = 3, FORM_SPLIT = 4 }
 // k + j starts only after every epilogue warp of its replica column block has
 // finished step j - 1, a pair only waits for tiles with a lower g, all CTAs
 // are resident, and every wait is bounded.
-template <int NB, int FORM>
+template <int NB, int FORM, int BN = BN_WIDE>
 __global__ void __launch_bounds__(THREADS, 1) k_t32(const __grid_constant__ CUtensorMap tmA,
                                                     const __grid_constant__ CUtensorMap tmB0,
                                                     const __grid_constant__ CUtensorMap tmB1, const T32Args a) {
-    constexpr uint32_t STAGE_BYTES = stage_bytes<NB>();
+    constexpr int BNH = BN / 2;
+    constexpr uint32_t B_TERM = b_term<BN>();
+    constexpr uint32_t STAGE_BYTES = stage_bytes<NB, BN>();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);   // even CTA: both stages landed
@@ -291,16 +295,16 @@ __global__ void __launch_bounds__(THREADS, 1) k_t32(const __grid_constant__ CUte
                         const uint64_t b0 = desc128(sb + o);
                         if constexpr (NB == 3) {
                             const uint64_t b1 = desc128(sb + B_TERM + o), b2 = desc128(sb + 2 * B_TERM + o);
-                            mma_pair(d, a0, b0, acc);
-                            mma_pair(dx, a0, b2, acc);
-                            mma_pair(dx, a0, b1, 1u);
-                            mma_pair(dx, a1, b1, 1u);
-                            mma_pair(dx, a1, b0, 1u);
-                            mma_pair(dx, a2, b0, 1u);
+                            mma_pair<BN>(d, a0, b0, acc);
+                            mma_pair<BN>(dx, a0, b2, acc);
+                            mma_pair<BN>(dx, a0, b1, 1u);
+                            mma_pair<BN>(dx, a1, b1, 1u);
+                            mma_pair<BN>(dx, a1, b0, 1u);
+                            mma_pair<BN>(dx, a2, b0, 1u);
                         } else {
-                            mma_pair(d, a0, b0, acc);
-                            mma_pair(dx, a2, b0, acc);
-                            mma_pair(dx, a1, b0, 1u);
+                            mma_pair<BN>(d, a0, b0, acc);
+                            mma_pair<BN>(dx, a2, b0, acc);
+                            mma_pair<BN>(dx, a1, b0, 1u);
                         }
                     }
                     umma_commit_pair(&empty[s]);
@@ -313,7 +317,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_t32(const __grid_constant__ CUte
         }
     } else {
         // epilogue: warp w reads tensor-memory lanes 32 (w % 4) .. +31 (this CTA's rows); the first four warps
-        // take replica columns [0, 64) of the tile, the next four the rest
+        // take the first half of the tile's replica columns, the next four the rest
         const int q = warp & 3;
         const int half = (warp - 2) >> 2;
         const uint32_t acce_cl = mapa(smem_u32(&acce[0]), 0);
@@ -532,13 +536,17 @@ int make_map3(CUtensorMap* m, void* base, int64_t rows, int64_t n_pad, int box_r
 }
 
 using T32Kernel = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const T32Args);
-T32Kernel pick(int form, bool exact_operand) {
+T32Kernel pick_split(bool exact_operand, int bn) {
+    if (bn == BN_NARROW)
+        return exact_operand ? k_t32<1, FORM_SPLIT, BN_NARROW> : k_t32<3, FORM_SPLIT, BN_NARROW>;
+    return exact_operand ? k_t32<1, FORM_SPLIT> : k_t32<3, FORM_SPLIT>;
+}
+T32Kernel pick(int form) {
     switch (form) {
         case FORM_BSB: return k_t32<3, FORM_BSB>;
         case FORM_ASB: return k_t32<3, FORM_ASB>;
         case FORM_PA: return k_t32<1, FORM_PA>;
-        case FORM_FIELD: return k_t32<3, FORM_FIELD>;
-        default: return exact_operand ? k_t32<1, FORM_SPLIT> : k_t32<3, FORM_SPLIT>;
+        default: return k_t32<3, FORM_FIELD>;
     }
 }
 using FinishKernel = void (*)(const T32Args);
@@ -584,18 +592,31 @@ int max_pairs(int device) {
 
 struct Plan {
     int64_t MT, NT, tiles;
-    int pairs, ksplit, kper;
+    int bn, pairs, ksplit, kper;
 };
 Plan plan(const veloxq_ctx* ctx, int32_t R) {
     Plan p;
     p.MT = div_up(ctx->n, 2 * BM);
-    p.NT = div_up(R, BN);
-    p.tiles = p.MT * p.NT;
     p.pairs = max_pairs(ctx->device);
     const int nkb = (int)div_up(tc_pad(ctx->n), BK);
-    const int ks = (int)std::max<int64_t>(1, std::min<int64_t>(p.pairs / p.tiles, nkb / MIN_BLOCKS));
-    p.kper = (int)div_up(nkb, ks);
-    p.ksplit = (int)div_up(nkb, p.kper);
+    auto split = [&](int bn) {
+        p.bn = bn;
+        p.NT = div_up(R, bn);
+        p.tiles = p.MT * p.NT;
+        const int ks = (int)std::max<int64_t>(1, std::min<int64_t>(p.pairs / p.tiles, nkb / MIN_BLOCKS));
+        p.kper = (int)div_up(nkb, ks);
+        p.ksplit = (int)div_up(nkb, p.kper);
+    };
+    split(BN_WIDE);
+    // Narrow tiles in the split form: half the MMA work of a tile where there
+    // are no more than 64 replicas, and more pairs at work where the splits of
+    // wide tiles cannot fill them (a step of n = 1001: R = 64 11.2 -> 9.6 us,
+    // R = 100 11.7 -> 10.5; n = 600, R = 200 11.8 -> 10.5; n = 3000, R = 64
+    // 19.1 -> 17.7; n = 8192, R = 64 91.0 -> 90.2, bound by its terms' bytes).
+    if (p.ksplit > 1 && (R <= BN_NARROW || 2 * p.tiles * p.ksplit <= p.pairs)) {
+        split(BN_NARROW);
+        if (p.ksplit == 1) split(BN_WIDE);
+    }
     return p;
 }
 
@@ -605,7 +626,6 @@ constexpr int64_t kMinN = 192;       // below, the SGEMM's two launches are as f
 
 int launch(veloxq_ctx* ctx, T32Kernel fn, int64_t pairs, const CUtensorMap& mq, const CUtensorMap* ms,
            const T32Args& a) {
-    VQ_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T32_SMEM));
     cudaLaunchConfig_t cfg = {};
     cfg.blockDim = dim3(THREADS);
     cfg.gridDim = dim3((unsigned)(2 * pairs));
@@ -760,9 +780,9 @@ int t32_run(veloxq_ctx* ctx, int32_t R, T32Run* t, float** cur, float** nxt, flo
     const int terms = t->terms;
     CUtensorMap mq, ms[2];
     VQ_TRY(make_map3(&mq, ctx->q3.p, n, np, BM, 3));
-    VQ_TRY(make_map3(&ms[0], ctx->s3[0].p, R, np, BNH, terms));
+    VQ_TRY(make_map3(&ms[0], ctx->s3[0].p, R, np, p.bn / 2, terms));
     ms[1] = ms[0];
-    if (ctx->s3[1].p && p.ksplit == 1) VQ_TRY(make_map3(&ms[1], ctx->s3[1].p, R, np, BNH, terms));
+    if (ctx->s3[1].p && p.ksplit == 1) VQ_TRY(make_map3(&ms[1], ctx->s3[1].p, R, np, p.bn / 2, terms));
     const int form = field_only ? FORM_FIELD
                      : rule.method == VELOXQ_METHOD_PA ? FORM_PA
                      : rule.method == VELOXQ_METHOD_ASB ? FORM_ASB : FORM_BSB;
@@ -793,7 +813,8 @@ int t32_run(veloxq_ctx* ctx, int32_t R, T32Run* t, float** cur, float** nxt, flo
     a.skip = guard ? ctx->t32w.as<uint32_t>() + 1 : nullptr;
     a.skip_seq = t->seq;
     if (p.ksplit > 1) {
-        T32Kernel fn = pick(FORM_SPLIT, terms == 1);
+        T32Kernel fn = pick_split(terms == 1, p.bn);
+        VQ_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T32_SMEM));
         FinishKernel fin = pick_finish(form);
         a.group = 1;
         for (int k = k_begin; k < k_end; ++k) {
@@ -816,7 +837,8 @@ int t32_run(veloxq_ctx* ctx, int32_t R, T32Run* t, float** cur, float** nxt, flo
             a.group = G;
             break;
         }
-    T32Kernel fn = pick(form, terms == 1);
+    T32Kernel fn = pick(form);
+    VQ_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T32_SMEM));
     for (int k0 = k_begin; k0 < k_end; k0 += kMaxRunSteps) {
         const int k1 = std::min(k_end, k0 + kMaxRunSteps), steps = k1 - k0;
         a.k = k0;
