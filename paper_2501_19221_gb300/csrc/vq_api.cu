@@ -277,12 +277,22 @@ int upload_schedule(veloxq_ctx* ctx, const RunParams& p) {
 veloxq_path choose_path(const veloxq_ctx* ctx, veloxq_path want, veloxq_prec prec, int32_t R) {
     if (want != VELOXQ_PATH_AUTO) return want;
     if (ctx->dense && prec != VELOXQ_PREC_FP32) return VELOXQ_PATH_DENSE;
-    if (ctx->dense) return resident_fits(ctx, R, nullptr, nullptr, nullptr) ? VELOXQ_PATH_RESIDENT : VELOXQ_PATH_DENSE;
+    // dense: the resident kernel while its couplings stay in shared memory,
+    // up to n = 512 then a step in the same order of sums (dense_ordered;
+    // n = 256 4.6 against 19.5 us, n = 512 11.4 against 78 us per step at 256
+    // replicas; at n = 200, on chip, the resident kernel takes 2.8 us)
+    if (ctx->dense) return resident_on_chip(ctx, R) ? VELOXQ_PATH_RESIDENT : VELOXQ_PATH_DENSE;
     // sparse: the resident kernel only when its couplings stay in shared
     // memory; when every CTA has to re-read them from L2 each step, the
     // streaming step is faster (Pegasus P_16: 84 against 29 us per step at
     // 1024 replicas, Zephyr Z_12: 228 against 29)
     return resident_on_chip(ctx, R) ? VELOXQ_PATH_RESIDENT : VELOXQ_PATH_STREAM;
+}
+
+// An instance of at most 512 variables on the dense path by the library's own
+// choice: its fields are summed as the resident kernel sums them.
+bool dense_ordered(const veloxq_ctx* ctx, const RunParams& p, veloxq_path path) {
+    return path == VELOXQ_PATH_DENSE && p.path == VELOXQ_PATH_AUTO && p.prec == VELOXQ_PREC_FP32 && ctx->has_csr;
 }
 
 int check_path(const veloxq_ctx* ctx, veloxq_path path, veloxq_prec prec, int32_t R) {
@@ -481,6 +491,8 @@ int enqueue_loop(veloxq_ctx* ctx, veloxq_path path, int32_t R, const RunParams& 
             VQ_TRY(t32_run(ctx, R, t32, &cur, &nxt, Y, at, k, k1 + 1, p.dt, p.a0, p.c0, nullptr, rule_of(p), false,
                            false));
             k = k1;
+        } else if (dense_ordered(ctx, p, path)) {
+            VQ_TRY(dense_step_ordered(ctx, R, cur, nxt, Y, at, k, p.dt, p.a0, p.c0, nullptr, rule_of(p)));
         } else if (path == VELOXQ_PATH_DENSE) {
             VQ_TRY(dense_step(ctx, R, cur, nxt, Y, at, k, p.dt, p.a0, p.c0, nullptr, rule_of(p)));
         } else {
@@ -738,7 +750,7 @@ int veloxq_solve(veloxq_ctx* ctx, int32_t replicas, int32_t steps, const veloxq_
         // the FP32 field in BF16 terms, unless the start state may leave their range
         T32Run t32r;
         bool use_t32 = false;
-        if (path == VELOXQ_PATH_DENSE && !use_tc) {
+        if (path == VELOXQ_PATH_DENSE && !use_tc && !dense_ordered(ctx, p, path)) {
             if (p.sigma0 == 0.0f || p.sigma0 >= 6.6174449e-24f /* 2^-77: |s| >= 2^-100 or 0 */)
                 VQ_TRY(t32_prepare(ctx, replicas, &use_t32));
             if (!use_t32) VQ_TRY(dense_prepare(ctx, replicas));
@@ -1119,7 +1131,8 @@ int veloxq_steps_dev(veloxq_ctx* ctx, int32_t R, int32_t k_begin, int32_t k_coun
     const int k_end = k_begin + k_count;
     T32Run t32r;
     bool t32 = false;
-    if (path == VELOXQ_PATH_DENSE && p.prec == VELOXQ_PREC_FP32) {
+    const bool ordered = dense_ordered(ctx, p, path);
+    if (path == VELOXQ_PATH_DENSE && p.prec == VELOXQ_PREC_FP32 && !ordered) {
         VQ_TRY(t32_prepare(ctx, R, &t32));
         if (t32) VQ_TRY(t32_split(ctx, R, S, rule_of(p), true, &t32r));
     }
@@ -1159,8 +1172,8 @@ int veloxq_steps_dev(veloxq_ctx* ctx, int32_t R, int32_t k_begin, int32_t k_coun
             return returns_early(ctx);
         }
         for (int k = k_begin; k < k_end; ++k) {
-            VQ_TRY(dense_step(ctx, R, cur, nxt, Y, at, k, p.dt, p.a0, p.c0, k == k_end - 1 ? F_last : nullptr,
-                              rule_of(p)));
+            VQ_TRY((ordered ? dense_step_ordered : dense_step)(ctx, R, cur, nxt, Y, at, k, p.dt, p.a0, p.c0,
+                                                               k == k_end - 1 ? F_last : nullptr, rule_of(p)));
             std::swap(cur, nxt);
         }
         return give_back();

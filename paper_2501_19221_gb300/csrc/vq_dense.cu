@@ -3,6 +3,7 @@
 // [R][n], Qoff symmetric row-major) with the ballistic-SB update fused into the
 // epilogue, and the exact readout energy in int64 fixed point.
 #include <algorithm>
+#include <type_traits>
 
 #include "vq_energy_mma.cuh"
 #include "vq_internal.cuh"
@@ -219,6 +220,165 @@ __global__ void __launch_bounds__(256) k_dense_finish(int32_t R, int32_t n, int 
     }
 }
 
+// The step of a dense instance of up to 512 variables whose couplings do not
+// fit the resident kernel's shared memory (n above about 230 for small
+// integers, 180 otherwise): the field is summed over j = 0 .. n - 1 without
+// i, one fused multiply-add after the other, which is the order of the
+// resident kernel's rows, so that a solve gives the same bits. A block takes
+// 32 variables x 16 replicas, a thread one variable of two replicas; Qoff's
+// 32 columns come to shared memory while the previous step still runs
+// (dependent launch), the replicas' rows behind it, in four stages of 128
+// variables. Bound by the latency of a warp's loads and sums while there is
+// one block per SM, by shared memory loads beyond. Per step, n = 256: 4.3 us
+// for 12 replicas, 4.6 for 256, 12.6 for 1024; n = 512: 7.3, 11.4 and 39.5 us.
+// The resident kernel, which reads the couplings from L2 there, one row per
+// thread, took 19.5 us at n = 256, 62 at n = 400 and 78 us at n = 512 (12 to
+// 256 replicas; 110 us for 1024). One or four replicas per warp: n = 512, 12
+// replicas 8.1 and 9.3 us, 1024 replicas 50 and 55 us.
+constexpr int OV = 32, OR = 16, OK = 128;   // variables and replicas of a block; variables of a stage
+constexpr int OW = 2, OT = 32 * OR / OW;    // replicas of a warp; threads of a block
+__host__ __device__ constexpr int ordered_pitch(int n) { return (n + 3) & ~3; }
+__device__ __forceinline__ void cp_async4(void* dst, const void* src, int bytes) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+                 "l"(src), "r"(bytes)
+                 : "memory");
+}
+template <bool SIGN>
+__global__ void __launch_bounds__(OT, 2) k_dense_ordered(int32_t R, int32_t n, const float* S_cur,
+                                                       const float* __restrict__ Qoff, float* S_nxt, float* Y,
+                                                       const float* __restrict__ bf, const float* __restrict__ a_table,
+                                                       int k, float dt, float a0, float c0, float* F_out, int method,
+                                                       float alpha, int wide) {
+    extern __shared__ __align__(16) float osm[];
+    float* qs = osm;                  // [n][OV]
+    const int pitch = ordered_pitch(n);
+    float* ss = osm + (size_t)n * OV;   // [OR][pitch]
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int tiles = (n + OV - 1) / OV;
+    const int n0 = (int)(blockIdx.x % tiles) * OV, r0 = (int)(blockIdx.x / tiles) * OR;
+    const int stages = (n + OK - 1) / OK;
+    for (int st = 0; st < 4; ++st) {
+        const int j0 = st * OK, j1 = min(n, j0 + OK);
+        if (wide) {                   // rows of Qoff 16-byte aligned
+            for (int e = tid; e < (j1 - j0) * (OV / 4); e += OT) {
+                const int j = j0 + e / (OV / 4), c = (e % (OV / 4)) * 4;
+                const int left = (n - (n0 + c)) * 4;
+                cp_async16(&qs[j * OV + c], left > 0 ? Qoff + (int64_t)j * n + n0 + c : Qoff, max(0, min(16, left)));
+            }
+        } else {
+            for (int e = tid; e < (j1 - j0) * OV; e += OT) {
+                const int j = j0 + e / OV, c = e % OV;
+                const bool in = n0 + c < n;
+                cp_async4(&qs[j * OV + c], in ? Qoff + (int64_t)j * n + n0 + c : Qoff, in ? 4 : 0);
+            }
+        }
+        cp_async_commit();
+    }
+    const int i = n0 + lane;
+    const float b = i < n ? __ldg(bf + i) : 0.0f, a_k = __ldg(a_table + k), lam = vqd::pa_lambda(a_k, a0);
+    // nothing the previous step wrote is read before this wait
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    for (int st = 0; st < 4; ++st) {
+        const int j0 = st * OK, len = max(0, min(n, j0 + OK) - j0);
+        if (wide) {
+            for (int e = tid; e < OR * (OK / 4); e += OT) {
+                const int r = e / (OK / 4), j = (e % (OK / 4)) * 4;
+                if (j >= len) continue;
+                const bool in = r0 + r < R;
+                cp_async16(&ss[r * pitch + j0 + j], in ? S_cur + (int64_t)(r0 + r) * n + j0 + j : S_cur, in ? 16 : 0);
+            }
+        } else {
+            for (int e = tid; e < OR * OK; e += OT) {
+                const int r = e / OK, j = e % OK;
+                if (j >= len) continue;
+                const bool in = r0 + r < R;
+                cp_async4(&ss[r * pitch + j0 + j], in ? S_cur + (int64_t)(r0 + r) * n + j0 + j : S_cur, in ? 4 : 0);
+            }
+        }
+        cp_async_commit();
+    }
+    const float* sw = ss + OW * w * pitch;   // this warp's replicas
+    float y[OW], acc[OW] = {};
+#pragma unroll
+    for (int u = 0; u < OW; ++u) {
+        const int r = r0 + OW * w + u;
+        y[u] = i < n && r < R ? __ldcg(Y + (int64_t)r * n + i) : 0.0f;
+    }
+    // eight variables at a time, the next eight's loads issued before the sums
+    struct Eight {
+        float q[8];
+        float4 s[OW][2];
+    } x0, x1;
+    auto load = [&](Eight& x, int j) {
+#pragma unroll
+        for (int t = 0; t < 8; ++t) x.q[t] = qs[(j + t) * OV + lane];
+#pragma unroll
+        for (int u = 0; u < OW; ++u) {
+            x.s[u][0] = *reinterpret_cast<const float4*>(sw + u * pitch + j);
+            x.s[u][1] = *reinterpret_cast<const float4*>(sw + u * pitch + j + 4);
+        }
+    };
+    auto sum = [&](const Eight& x, int j, auto own) {
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+#pragma unroll
+            for (int u = 0; u < OW; ++u) {
+                const float4 v4 = x.s[u][t / 4];
+                float v = t % 4 == 0 ? v4.x : t % 4 == 1 ? v4.y : t % 4 == 2 ? v4.z : v4.w;
+                if constexpr (SIGN) v = vqd::pa_sign(v);
+                const float f = fmaf(x.q[t], v, acc[u]);
+                acc[u] = own && j + t == i ? acc[u] : f;
+            }
+        }
+    };
+    auto sum8 = [&](const Eight& x, int j) {
+        if (j >= n0 && j < n0 + OV) sum(x, j, std::true_type{});   // the block's own variables (n0 and j are multiples of 8)
+        else sum(x, j, std::false_type{});
+    };
+    for (int st = 0; st < stages; ++st) {
+        // the states of later stages may still be on their way
+        if (st == 0) cp_async_wait<3>();
+        else if (st == 1) cp_async_wait<2>();
+        else if (st == 2) cp_async_wait<1>();
+        else cp_async_wait<0>();
+        __syncthreads();
+        const int j1 = min(n, (st + 1) * OK), j8 = j1 & ~7;
+        int j = st * OK;
+        if (j < j8) load(x0, j);
+#pragma unroll 1
+        for (; j < j8; j += 16) {
+            if (j + 8 < j8) load(x1, j + 8);
+            sum8(x0, j);
+            if (j + 8 >= j8) break;
+            if (j + 16 < j8) load(x0, j + 16);
+            sum8(x1, j + 8);
+        }
+        for (j = j8; j < j1; ++j) {
+            if (j == i) continue;
+#pragma unroll
+            for (int u = 0; u < OW; ++u) {
+                float v = sw[u * pitch + j];
+                if constexpr (SIGN) v = vqd::pa_sign(v);
+                acc[u] = fmaf(qs[j * OV + lane], v, acc[u]);
+            }
+        }
+    }
+    cp_async_wait<0>();
+    if (i >= n) return;
+#pragma unroll
+    for (int u = 0; u < OW; ++u) {
+        const int r = r0 + OW * w + u;
+        if (r >= R) break;
+        const int64_t p = (int64_t)r * n + i;
+        if (F_out) F_out[p] = acc[u];
+        float s = sw[u * pitch + i];
+        vqd::step_update(method, acc[u], b, a_k, lam, dt, a0, c0, alpha, s, y[u]);
+        S_nxt[p] = s;
+        Y[p] = y[u];
+    }
+}
+
 // Exact energy of x_r = [S_r > 0] (or of a caller batch of bytes), fixed
 // point: parts[g][r] = sum over the 64 rows of tile g of
 // x_ri (dfix_i + sum_{j != i} qfix(Q_ij) x_rj), Q as given. One block per
@@ -324,6 +484,19 @@ int launch_dense_energy(veloxq_ctx* ctx, int64_t R, const float* S, const uint8_
 int dense_step(veloxq_ctx* ctx, int32_t R, const float* S_cur, float* S_nxt, float* Y, const float* a_table, int k,
                float dt, float a0, float c0, float* F_out, const Rule& rule) {
     return launch_dense_step<false>(ctx, R, S_cur, S_nxt, Y, a_table, k, dt, a0, c0, F_out, rule);
+}
+
+int dense_step_ordered(veloxq_ctx* ctx, int32_t R, const float* S_cur, float* S_nxt, float* Y, const float* a_table,
+                       int k, float dt, float a0, float c0, float* F_out, const Rule& rule) {
+    const int32_t n = (int32_t)ctx->n;
+    auto bytes = [](int m) { return sizeof(float) * ((size_t)m * OV + (size_t)OR * ordered_pitch(m)); };
+    const dim3 g((unsigned)(div_up(n, OV) * div_up(R, OR)));
+    auto fn = rule.method == VELOXQ_METHOD_PA ? k_dense_ordered<true> : k_dense_ordered<false>;
+    VQ_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes(512)));
+    const int wide = n % 4 == 0 && ((reinterpret_cast<uintptr_t>(ctx->qoff32.p) | reinterpret_cast<uintptr_t>(S_cur)) & 15) == 0;
+    VQ_CUDA(launch_dependent(true, fn, g, dim3(OT), bytes(n), ctx->stream, R, n, S_cur, ctx->qoff32.as<float>(), S_nxt, Y,
+                             ctx->bf.as<float>(), a_table, k, dt, a0, c0, F_out, rule.method, rule.alpha, wide));
+    return VELOXQ_OK;
 }
 
 int dense_prepare(veloxq_ctx* ctx, int32_t R) {

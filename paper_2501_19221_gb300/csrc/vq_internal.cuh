@@ -237,6 +237,9 @@ int resident_run(veloxq_ctx* ctx, int32_t R, const RunParams& p, uint64_t seed, 
 // dense kernels (vq_dense.cu)
 int dense_step(veloxq_ctx* ctx, int32_t R, const float* S_cur, float* S_nxt, float* Y,
                const float* a_table, int k, float dt, float a0, float c0, float* F_out, const Rule& rule = Rule());
+// the step of dense instances of at most 512 variables beyond the resident kernel, in its order of sums
+int dense_step_ordered(veloxq_ctx* ctx, int32_t R, const float* S_cur, float* S_nxt, float* Y, const float* a_table,
+                       int k, float dt, float a0, float c0, float* F_out, const Rule& rule);
 // only (or null): the kernels do nothing unless *only == only_seq
 int dense_field(veloxq_ctx* ctx, int32_t R, const float* S, float* F, const uint32_t* only = nullptr,
                 uint32_t only_seq = 0);
