@@ -47,18 +47,15 @@ L2_FLUSH_BYTES = 256 << 20          # > 129 MB of L2
 # changes after its capture must be removed from this table.
 NCU_TRAFFIC = {
     ("k_resident", "chimera_c16"): 282_624,
-    ("k_stream_step", "lattice_l100"): 4_104_791_000,
+    ("k_stream_step", "lattice_l100"): 4_102_344_192,
     ("k_stream_step", "hubo_chain_1e7"): 3_555_804_000,
-    ("k_stream_step", "xorsat_3r3x_1e5"): 846_672_128,
-    ("k_stream_step", "tile_planting_l300"): 314_659_499,
     ("k_adj_a+k_adj_b", "grad_l100"): 9_577_706_240,
-    ("k_tc_step", "sk_n8192_fp8"): 291_477_740,     # per step: one 200-step launch, 58.30 GB / 200
+    ("k_tc_step", "sk_n8192_fp8"): 290_595_539,     # per step: one 200-step launch, 58.12 GB / 200
     ("k_tc_step", "sk_n8192_bf16"): 435_910_845,    # per step: one 200-step launch, 87.18 GB / 200
     ("k_batch", "wishart_b512_k20"): 45_369_958_000,
     ("k_batch", "wishart_b512_k20_fp8"): 29_200_151_000,
 }
 SMEM_BYTES_PER_CLK_PER_SM = 128     # 32 banks x 4 bytes
-FP32_LANES_PER_SM = 128
 PREC_NAMES = {0: "fp32", 1: "bf16", 2: "fp8", 3: "fp8_one_term"}
 
 
@@ -163,7 +160,7 @@ def workload(name: str, for_oracle: bool = False) -> dict:
         Q, c = I.sk_qubo(8192, seed=0)
         form = name[len("sk_n8192_"):]
         prec = {"fp32": 0, "bf16": 1, "fp8": 2, "fp8_one_term": 3}[form]
-        what = {"fp32": "FP32 (CUDA cores)", "bf16": "BF16 (tensor cores)",
+        what = {"fp32": "FP32 accuracy (tensor cores, three BF16 terms per operand)", "bf16": "BF16 (tensor cores)",
                 "fp8": "FP8 E4M3 (tensor cores; per-row scales for Qoff, S as two E4M3 terms)",
                 "fp8_one_term": "FP8 E4M3 (tensor cores; per-row scales for Qoff, S as one E4M3 term)"}[form]
         return {"name": name, "kind": "dense", "Q": Q, "c": c, "n": 8192, "R": 1024, "K": 200,
@@ -552,7 +549,7 @@ def roofline(B, w, runner, path, main_ms, main_launches):
     if path == B.VELOXQ_PATH_DENSE and w.get("prec", 0) in (1, 2, 3):
         return tc_roofline(w["prec"], w.get("method", "bsb"), n, R, main_ms / K)
     if path == B.VELOXQ_PATH_DENSE:
-        return sgemm_roofline(n, R, main_ms / K)
+        return fp32_roofline(n, R, w.get("method", "bsb"), main_ms / K)
     # state r/w + couplings (int8 2Qs or float Qs) and int32 columns, per step; the row
     # pointers are read only when rows differ in length (rows of equal length start at i * degree)
     per_nnz = 5 if runner.int8_couplings else 8
@@ -584,19 +581,19 @@ def tc_roofline(prec, method, n, R, per_ms):
             "ms_per_launch": per_ms}
 
 
-def sgemm_roofline(n, R, per_ms):
-    """Roofline of one FP32 CUDA-core step (k_dense_step, plus k_dense_finish
-    when the k-loop is split): 2 n^2 R FLOP against the FP32 FMA peak derived
-    from the lane count and the maximum clock."""
+def fp32_roofline(n, R, method, per_ms):
+    """Roofline of one FP32-accurate step on the tensor cores (k_t32, and
+    k_t32_finish when the k-loop is split): six BF16 products of 2 n^2 R FLOP
+    (three for Parallel Annealing, whose operand is one exact term) against
+    the measured BF16 peak."""
     peaks, src = _peaks()
-    sms = num_sms()
-    flops = 2.0 * n * n * R
-    fp32_peak = sms * FP32_LANES_PER_SM * 2 * peaks.get("sm_max_mhz", 2070.0) * 1e6 / 1e12
+    terms = 3 if method == "pa" else 6
+    flops = 2.0 * n * n * R * terms
     ach = flops / (per_ms / 1e3) / 1e12
-    return {"kernel": "k_dense_step", "bound": "alu", "achieved": ach, "peak": fp32_peak, "unit": "TFLOP/s",
-            "frac": ach / fp32_peak, "traffic": None,
-            "peak_source": f"derived: {sms} SMs x {FP32_LANES_PER_SM} FP32 lanes x 2 (FMA) x {src} max clock",
-            "algorithmic_flops_per_launch": flops, "ms_per_launch": per_ms}
+    return {"kernel": "k_t32", "bound": "tensor", "achieved": ach, "peak": peaks["bf16_tflops"], "unit": "TFLOP/s",
+            "frac": ach / peaks["bf16_tflops"], "traffic": None, "peak_source": f"{src} bf16_tflops",
+            "algorithmic_flops_per_launch": flops, "flops_per_launch_note": f"{terms} BF16 products per step",
+            "ms_per_launch": per_ms}
 
 
 def field_errors(B, stream, Q, R=1024, rows=96, seed=7):
@@ -637,8 +634,9 @@ def time_to_target(B, stream, seeds=32, n=8192, R=1024, K=200, method=0):
     construction); a form reaches it at the smallest K' of TTT_GRID where at
     least half of the seeds end at or below E*. Times are CUDA-event times of
     whole solves (median over the seeds). The FP32 form's step is also given
-    as its own roofline fraction (the SGEMM against the FP32 FMA peak), so
-    that the ratios can be read against the quality of the baseline kernel."""
+    as its own roofline fraction (its six BF16 products, three for Parallel
+    Annealing, against the BF16 peak), so that the ratios can be read against
+    the quality of the baseline kernel."""
     import torch
     Q, c = I.sk_qubo(n, seed=0)
     ctx = B.veloxq_create_dense(Q, c)
@@ -665,10 +663,10 @@ def time_to_target(B, stream, seeds=32, n=8192, R=1024, K=200, method=0):
         E_star = float(np.median([e for e, _ in fp32]))
         t32 = float(np.median([t for _, t in fp32]))
         out["E_star"] = E_star
-        sg = sgemm_roofline(n, R, float(np.median(steps_ms)) / K)
+        sg = fp32_roofline(n, R, mname, float(np.median(steps_ms)) / K)
         out["fp32"] = {"steps": K, "ms": t32, "success": float(np.mean([e <= E_star for e, _ in fp32])),
                        "step_ms": sg["ms_per_launch"], "step_tflops": sg["achieved"],
-                       "step_frac_of_fp32_peak": sg["frac"], "step_peak_source": sg["peak_source"]}
+                       "step_frac_of_bf16_peak": sg["frac"], "step_peak_source": sg["peak_source"]}
         # Parallel Annealing's operand is exact in one E4M3 term: FP8 and FP8_ONE_TERM are the same run
         arms = [("bf16", 1), ("fp8", 2)] + ([] if method == 2 else [("fp8_one_term", 3)])
         for name, prec in arms:

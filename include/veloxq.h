@@ -68,9 +68,15 @@ typedef enum {
 /* Element type of a coupling array passed in. */
 typedef enum { VELOXQ_I8 = 0, VELOXQ_I32 = 1, VELOXQ_F32 = 2, VELOXQ_F64 = 3 } veloxq_vtype;
 
-/* Operand precision of the dense local-field product F = Qoff S. FP32 runs on
- * the CUDA cores; the others run on the tcgen05 tensor cores; all accumulate
- * in FP32. Sparse contexts always use FP32 (or exact int8 couplings).
+/* Operand precision of the dense local-field product F = Qoff S. All run on
+ * the tcgen05 tensor cores and accumulate in FP32. Sparse contexts always use
+ * FP32 (or exact int8 couplings).
+ *   FP32:          every operand as the exact sum of three BF16 terms, the six
+ *                  term products down to 2^-16 of the leading one (error
+ *                  against FP64 below that of an FP32 sum of products); small
+ *                  n, and values whose terms would leave BF16's range (not
+ *                  finite, |x| >= 2^127, 0 < |x| < 2^-100), as FP32 sums of
+ *                  products on the CUDA cores.
  *   BF16:          bf16(Qoff) x bf16(s).
  *   FP8:           Qoff as E4M3 with one FP32 scale per row (amax_i / 448);
  *                  S (whose entries the walls keep in [-1, 1]) with the fixed
@@ -96,9 +102,10 @@ typedef enum {
 
 /* Kernel path selection. VELOXQ_PATH_AUTO picks by size and format: BF16 and
  * FP8 on dense contexts take the dense path; FP32 on dense contexts the
- * resident kernel when it fits, else the dense path; sparse contexts the
- * resident kernel when its couplings fit in shared memory, else the
- * streaming path. */
+ * resident kernel when its couplings fit in shared memory, else the dense
+ * path (up to n = 512 with the resident kernel's order of sums, so that both
+ * give the same bits); sparse contexts the resident kernel when its couplings
+ * fit in shared memory, else the streaming path. */
 typedef enum {
     VELOXQ_PATH_AUTO = 0,
     VELOXQ_PATH_RESIDENT = 1,  /* sparse rows, whole run in one launch, state in shared memory */
