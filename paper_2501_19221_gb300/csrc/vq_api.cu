@@ -698,7 +698,11 @@ int veloxq_solve(veloxq_ctx* ctx, int32_t replicas, int32_t steps, const veloxq_
     if (E_best_int && !ctx->integer) return fail(VELOXQ_EINVAL, "E_best_int requires an integer-valued context");
     RunParams p;
     VQ_TRY(resolve(ctx, sched, steps, &p));
-    const veloxq_path path = choose_path(ctx, p.path, p.prec, replicas);
+    veloxq_path path = choose_path(ctx, p.path, p.prec, replicas);
+    // a captured loop holds a node per step: the longest runs stay in the
+    // resident kernel's one launch (the same bits)
+    if (dense_ordered(ctx, p, path) && steps > (1 << 20) && resident_fits(ctx, replicas, nullptr, nullptr, nullptr))
+        path = VELOXQ_PATH_RESIDENT;
     VQ_TRY(check_path(ctx, path, p.prec, replicas));
     ctx->batch_R = 0;
     CtxExtra* ex = extra(ctx);
@@ -772,6 +776,7 @@ int veloxq_solve(veloxq_ctx* ctx, int32_t replicas, int32_t steps, const veloxq_
                                      (uint64_t)(uintptr_t)ctx->res.p, (uint64_t)(uintptr_t)ctx->best_bits.p,
                                      (uint64_t)(uintptr_t)ctx->flags.p, (uint64_t)(uintptr_t)ctx->a_table.p};
         key.push_back((uint64_t)p.method);
+        key.push_back((uint64_t)dense_ordered(ctx, p, path));
         for (uint64_t v : {(uint64_t)tc_e, (uint64_t)ctx->eplanes, (uint64_t)(uintptr_t)ctx->eplane.p,
                            (uint64_t)(uintptr_t)ctx->exop.p, (uint64_t)(uintptr_t)ctx->efield.p,
                            (uint64_t)use_t32, (uint64_t)(uintptr_t)ctx->q3.p, (uint64_t)(uintptr_t)ctx->s3[0].p,

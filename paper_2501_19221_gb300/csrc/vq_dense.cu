@@ -221,8 +221,8 @@ __global__ void __launch_bounds__(256) k_dense_finish(int32_t R, int32_t n, int 
 }
 
 // The step of a dense instance of up to 512 variables whose couplings do not
-// fit the resident kernel's shared memory (n above about 230 for small
-// integers, 180 otherwise): the field is summed over j = 0 .. n - 1 without
+// fit the resident kernel's shared memory (n above about 235 for small
+// integers, 190 otherwise): the field is summed over j = 0 .. n - 1 without
 // i, one fused multiply-add after the other, which is the order of the
 // resident kernel's rows, so that a solve gives the same bits. A block takes
 // 32 variables x 16 replicas, a thread one variable of two replicas; Qoff's

@@ -52,3 +52,17 @@ def test_same_bits_as_resident(B, n, R, whole, method):
     assert np.array_equal(a["x"], b["x"]) and a["E"] == b["E"]
     assert np.array_equal(a["E_per_replica"], b["E_per_replica"])
     assert all(torch.equal(x, y) for x, y in zip(ta, tb))
+
+
+@pytest.mark.parametrize("n,sigma0", [(320, 0.1), (256, 1e-30)])     # asked for: tensor cores; SGEMM
+def test_chosen_and_asked_dense_path_take_turns(B, n, sigma0):
+    """The captured loop of one is not replayed for the other: each solve launches what it launches on a new context
+    and gives that context's energies."""
+    ctx = _ctx(B, n, False)
+    for path in (AUTO, DENSE, AUTO, DENSE):
+        sched = B.make_schedule(readout_every=20, path=path, sigma0=sigma0)
+        new = _ctx(B, n, False)
+        a, b = (B.veloxq_solve(c, 17, 60, sched, seed=2) for c in (ctx, new))
+        assert B.veloxq_last_timing(ctx).path == DENSE
+        assert B.veloxq_last_timing(ctx).launches == B.veloxq_last_timing(new).launches
+        assert np.array_equal(a["E_per_replica"], b["E_per_replica"])
