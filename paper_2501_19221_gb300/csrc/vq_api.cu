@@ -446,6 +446,15 @@ int returns_early(veloxq_ctx* ctx) {
     return VELOXQ_OK;
 }
 
+// For an entry point that leaves kernels on the context's scratch behind when
+// it returns, on whichever of its exits: records the event there.
+struct EarlyReturn {
+    veloxq_ctx* ctx;
+    ~EarlyReturn() {
+        if (ctx) returns_early(ctx);
+    }
+};
+
 int check_err_word(veloxq_ctx* ctx) {
     int h = 0;
     VQ_CUDA(cudaMemcpyAsync(&h, ctx->errw.p, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
@@ -1090,6 +1099,9 @@ int veloxq_field_dev(veloxq_ctx* ctx, int32_t R, veloxq_prec prec, const float* 
     VQ_TRY(check_device(ctx));
     if (R < 1 || R > kMaxReplicas || !S || !F) return fail(VELOXQ_EINVAL, "R in [1, 2^20] and non-NULL S, F required");
     if (prec < VELOXQ_PREC_FP32 || prec > VELOXQ_PREC_FP8_ONE_TERM) return fail(VELOXQ_EINVAL, "unknown precision");
+    if (!ctx->dense && prec != VELOXQ_PREC_FP32)
+        return fail(VELOXQ_EUNSUPPORTED, "sparse contexts run the field in FP32 (or exact int8)");
+    EarlyReturn early{ctx};
     if (ctx->dense) {
         if (prec == VELOXQ_PREC_FP32) {
             bool t32 = false;
@@ -1100,18 +1112,15 @@ int veloxq_field_dev(veloxq_ctx* ctx, int32_t R, veloxq_prec prec, const float* 
             T32Run t;
             VQ_TRY(t32_split(ctx, R, S, Rule(), true, &t));
             VQ_TRY(t32_run(ctx, R, &t, nullptr, nullptr, nullptr, nullptr, 0, 1, 0.f, 0.f, 0.f, F, Rule(), true, true));
-            VQ_TRY(dense_field(ctx, R, S, F, ctx->t32w.as<uint32_t>() + 1, t.seq));
-            return returns_early(ctx);
+            return dense_field(ctx, R, S, F, ctx->t32w.as<uint32_t>() + 1, t.seq);
         }
         TcRun tc;
         VQ_TRY(tc_setup(ctx, prec, R, &tc));
         VQ_TRY(async_words(ctx));
         VQ_TRY(tc_quant_s(ctx, prec, R, S, tc.sop[0]));
-        VQ_TRY(tc_field(ctx, prec, R, tc.mq, tc.ms[0], tc.lo(0), F, ctx->t32w.as<int>(),
-                        static_cast<int*>(ctx->t32h.dev)));
-        return returns_early(ctx);
+        return tc_field(ctx, prec, R, tc.mq, tc.ms[0], tc.lo(0), F, ctx->t32w.as<int>(),
+                        static_cast<int*>(ctx->t32h.dev));
     }
-    if (prec != VELOXQ_PREC_FP32) return fail(VELOXQ_EUNSUPPORTED, "sparse contexts run the field in FP32 (or exact int8)");
     const int64_t nR = ctx->n * (int64_t)R;
     VQ_TRY(ctx->s_a.ensure(sizeof(float) * nR));
     VQ_TRY(ctx->f.ensure(sizeof(float) * nR));
@@ -1134,6 +1143,8 @@ int veloxq_steps_dev(veloxq_ctx* ctx, int32_t R, int32_t k_begin, int32_t k_coun
     VQ_TRY(check_path(ctx, path, p.prec, R));
     const int64_t n = ctx->n, nR = n * (int64_t)R;
     const int k_end = k_begin + k_count;
+    // the resident kernel works in S and Y alone
+    EarlyReturn early{path == VELOXQ_PATH_RESIDENT ? nullptr : ctx};
     T32Run t32r;
     bool t32 = false;
     const bool ordered = dense_ordered(ctx, p, path);
@@ -1161,8 +1172,7 @@ int veloxq_steps_dev(veloxq_ctx* ctx, int32_t R, int32_t k_begin, int32_t k_coun
         if (t32) {
             VQ_TRY(t32_run(ctx, R, &t32r, &cur, &nxt, Y, at, k_begin, k_end, p.dt, p.a0, p.c0, F_last, rule_of(p), false,
                            false));
-            VQ_TRY(give_back());
-            return returns_early(ctx);
+            return give_back();
         }
         if (p.prec != VELOXQ_PREC_FP32) {
             TcRun tc;
@@ -1173,8 +1183,7 @@ int veloxq_steps_dev(veloxq_ctx* ctx, int32_t R, int32_t k_begin, int32_t k_coun
             VQ_TRY(tc_run(ctx, p.prec, R, tc.mq, tc.ms, tc.lo(), 0, cur, nxt, Y, tc.sop, at, k_begin, k_end, p.dt,
                           p.a0, p.c0, F_last, ctx->t32w.as<int>(), rule_of(p), static_cast<int*>(ctx->t32h.dev)));
             if (k_count & 1) std::swap(cur, nxt);
-            VQ_TRY(give_back());
-            return returns_early(ctx);
+            return give_back();
         }
         for (int k = k_begin; k < k_end; ++k) {
             VQ_TRY((ordered ? dense_step_ordered : dense_step)(ctx, R, cur, nxt, Y, at, k, p.dt, p.a0, p.c0,

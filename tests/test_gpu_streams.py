@@ -1,0 +1,103 @@
+"""Calls on one context from several streams. A call that returns before its
+kernels end leaves them on the context's scratch (the second state buffer,
+operand copies, partial fields, transposed states), so a call on another
+stream is ordered behind it. The first stream is held up by a timed sleep:
+when the second call's work has ended, the first call's must have ended too."""
+import numpy as np
+import pytest
+
+from paper_2501_19221_gb300 import instances as I
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+HOLD = 100_000_000        # SM cycles, about 50 ms
+STREAM, DENSE = 2, 3
+
+
+@pytest.fixture(scope="module")
+def B():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    import __graft_entry__ as g
+    g.build()
+    from paper_2501_19221_gb300 import binding
+    return binding
+
+
+def _dense(B, n):
+    J, _ = I.sk_qubo(n, seed=n)
+    return B.veloxq_create_ising_dense(J), n
+
+
+def _sparse(B):
+    sp = I.chimera_ising(4, 4, 4, seed=1)
+    return B.veloxq_create_ising_csr(sp.n, sp.rowptr, sp.col, sp.val, sp.lin), sp.n
+
+
+def _state(R, n, seed):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    return torch.rand(R, n, generator=g, device="cuda") * 2 - 1, torch.rand(R, n, generator=g, device="cuda") * 2 - 1
+
+
+# the exits of a step call: in the resident kernel's order of sums, FP32 sums of products, FP32 tensor-core form,
+# BF16, and sparse rows
+STEPS = [("ordered", 300, {}), ("sgemm", 150, {"path": DENSE}), ("terms", 300, {"path": DENSE}),
+         ("bf16", 300, {"prec": 1}), ("rows", 0, {"path": STREAM})]
+
+
+@pytest.mark.parametrize("form,n,kw", STEPS, ids=[s[0] for s in STEPS])
+def test_steps_on_two_streams(B, form, n, kw):
+    ctx, n = _dense(B, n) if n else _sparse(B)
+    R, odd = 17, 5
+    sched = B.make_schedule(c0=1.0, **kw)
+
+    def steps(S, Y):
+        B.veloxq_steps_dev(ctx, R, 0, odd, 20, sched, S, Y)
+
+    want = []
+    for seed in (1, 2):                              # in turn (and everything allocated, the schedule uploaded)
+        S, Y = _state(R, n, seed)
+        steps(S, Y)
+        torch.cuda.synchronize()
+        want += [S, Y]
+    (S1, Y1), (S2, Y2) = _state(R, n, 1), _state(R, n, 2)
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s1):
+        if form != "terms":                          # that form waits for its stream (the range of S)
+            torch.cuda._sleep(HOLD)
+        steps(S1, Y1)
+        e1 = s1.record_event()
+    with torch.cuda.stream(s2):
+        steps(S2, Y2)
+        e2 = s2.record_event()
+    e2.synchronize()
+    assert e1.query()
+    assert all(torch.equal(a, b) for a, b in zip(want, (S1, Y1, S2, Y2)))
+
+
+@pytest.mark.parametrize("n,prec", [(150, 0), (300, 0), (300, 1), (0, 0)])
+def test_fields_on_two_streams(B, n, prec):
+    ctx, n = _dense(B, n) if n else _sparse(B)
+    R = 17
+    S, _ = _state(R, n, 1)
+    want, got = [], []
+    for x in (S, -S):
+        F = torch.empty_like(S)
+        B.veloxq_field_dev(ctx, R, prec, x, F)
+        torch.cuda.synchronize()
+        want.append(F)
+    streams, ends = [torch.cuda.Stream(), torch.cuda.Stream()], []
+    xs = [S, -S]
+    got = [torch.empty_like(S), torch.empty_like(S)]
+    torch.cuda.synchronize()
+    for q, st in enumerate(streams):
+        with torch.cuda.stream(st):
+            if q == 0:
+                torch.cuda._sleep(HOLD)
+            B.veloxq_field_dev(ctx, R, prec, xs[q], got[q])
+            ends.append(st.record_event())
+    ends[1].synchronize()
+    assert ends[0].query()
+    assert all(torch.equal(a, b) for a, b in zip(want, got))
