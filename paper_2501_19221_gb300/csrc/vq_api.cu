@@ -172,9 +172,11 @@ struct CtxExtra {
     int tune_stages = 0, tune_split = 0;   // form of the last batched launch headed by this context
     BatchGraph bgraph;                     // its captured device part
     // the last call that returned before its kernels ended: recorded behind
-    // them, waited for by a call on another stream (they share the scratch)
+    // them, waited for by every later call on another stream (they share the
+    // scratch); streams are told apart by their id, since a handle may be
+    // reused or (per-thread default stream) stand for several
     cudaEvent_t aev = nullptr;
-    cudaStream_t astream = nullptr;
+    unsigned long long astream = 0;
     bool apending = false;
     ~CtxExtra() {
         if (graph) cudaGraphExecDestroy(graph);
@@ -413,6 +415,29 @@ void tune_store(const std::string& key, int stages, int group) {
     }
 }
 
+// Orders `stream` behind the kernels that a call on another stream left on the
+// context's scratch. A stream in capture takes no event from outside: the host
+// waits for them instead (a replay may follow at any time).
+int order_behind_pending(veloxq_ctx* ctx, cudaStream_t stream) {
+    CtxExtra* ex = extra(ctx);
+    if (!ex || !ex->apending) return VELOXQ_OK;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    VQ_CUDA(cudaStreamIsCapturing(stream, &cs));
+    if (cs == cudaStreamCaptureStatusNone) {
+        unsigned long long id = 0;
+        VQ_CUDA(cudaStreamGetId(stream, &id));
+        if (id != ex->astream) VQ_CUDA(cudaStreamWaitEvent(stream, ex->aev, 0));
+        return VELOXQ_OK;
+    }
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;   // this wait is no part of any capture
+    VQ_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
+    const cudaError_t e = cudaEventSynchronize(ex->aev);
+    VQ_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
+    VQ_CUDA(e);
+    ex->apending = false;
+    return VELOXQ_OK;
+}
+
 // Every call on a context runs on the device the context was created on,
 // which must be the current device: its buffers live there.
 // A bounded wait that gave up in an earlier asynchronous call is reported here.
@@ -422,15 +447,7 @@ int check_device(veloxq_ctx* ctx) {
     if (dev != ctx->device)
         return fail(VELOXQ_EINVAL, "the context was created on device " + std::to_string(ctx->device) +
                                        ", which must be the current device (current: " + std::to_string(dev) + ")");
-    CtxExtra* ex = extra(ctx);
-    if (ex && ex->apending && ex->astream != ctx->stream) {
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        VQ_CUDA(cudaStreamIsCapturing(ctx->stream, &cs));
-        if (cs == cudaStreamCaptureStatusNone) {
-            VQ_CUDA(cudaStreamWaitEvent(ctx->stream, ex->aev, 0));
-            ex->apending = false;
-        }
-    }
+    VQ_TRY(order_behind_pending(ctx, ctx->stream));
     return t32_check(ctx);
 }
 
@@ -440,8 +457,8 @@ int returns_early(veloxq_ctx* ctx) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     VQ_CUDA(cudaStreamIsCapturing(ctx->stream, &cs));
     if (!ex || cs != cudaStreamCaptureStatusNone) return VELOXQ_OK;
+    VQ_CUDA(cudaStreamGetId(ctx->stream, &ex->astream));
     VQ_CUDA(cudaEventRecord(ex->aev, ctx->stream));
-    ex->astream = ctx->stream;
     ex->apending = true;
     return VELOXQ_OK;
 }

@@ -101,3 +101,52 @@ def test_fields_on_two_streams(B, n, prec):
     ends[1].synchronize()
     assert ends[0].query()
     assert all(torch.equal(a, b) for a, b in zip(want, got))
+
+
+def _held_steps(ctx, B, stream, R, S, Y, sched):
+    """A step call behind the sleep; its end as an event."""
+    with torch.cuda.stream(stream):
+        torch.cuda._sleep(HOLD)
+        B.veloxq_steps_dev(ctx, R, 0, 1, 20, sched, S, Y)
+        return stream.record_event()
+
+
+def test_third_stream_waits_too(B):
+    """A call in between that leaves nothing on the scratch does not end the wait for the first one."""
+    ctx, n = _dense(B, 300)
+    R, sched = 17, B.make_schedule(c0=1.0)
+    states = [_state(R, n, s) for s in (1, 2, 3)]
+    B.veloxq_steps_dev(ctx, R, 0, 1, 20, sched, *_state(R, n, 1))
+    torch.cuda.synchronize()
+    s1, s2, s3 = (torch.cuda.Stream() for _ in range(3))
+    e1 = _held_steps(ctx, B, s1, R, *states[0], sched)
+    with torch.cuda.stream(s2):
+        B.veloxq_init_state_dev(ctx, R, 1, 0.1, *states[1])
+    with torch.cuda.stream(s3):
+        B.veloxq_steps_dev(ctx, R, 0, 1, 20, sched, *states[2])
+        e3 = s3.record_event()
+    e3.synchronize()
+    assert e1.query()
+
+
+def test_captured_call_waits_at_capture(B):
+    ctx, n = _dense(B, 300)
+    R, sched = 17, B.make_schedule(c0=1.0)
+    S, F = _state(R, n, 1)[0], torch.empty(R, n, device="cuda")
+    B.veloxq_field_dev(ctx, R, 0, S, F)              # buffers, so that the capture allocates nothing
+    want = F.clone()
+    X, Y = _state(R, n, 2)
+    B.veloxq_steps_dev(ctx, R, 0, 1, 20, sched, X, Y)
+    torch.cuda.synchronize()
+    F.zero_()
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    e1 = _held_steps(ctx, B, s1, R, X, Y, sched)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(s2):
+        graph.capture_begin()
+        B.veloxq_field_dev(ctx, R, 0, S, F)
+        graph.capture_end()
+        assert e1.query()
+        graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(F, want)
