@@ -940,6 +940,7 @@ int veloxq_solve_batch(veloxq_ctx* const* ctxs, int32_t count, int32_t replicas,
     CtxExtra* ex = extra(c0);
     cudaStream_t st = ex->work;
     for (int32_t m = 0; m < count; ++m) {
+        VQ_TRY(order_behind_pending(ctxs[m], st));   // steps left on another stream than the context's
         if (m > 0 && ctxs[m]->stream == ctxs[m - 1]->stream) continue;   // ordered already
         VQ_CUDA(cudaEventRecord(ex->ev, ctxs[m]->stream));
         VQ_CUDA(cudaStreamWaitEvent(st, ex->ev, 0));

@@ -150,3 +150,31 @@ def test_captured_call_waits_at_capture(B):
         graph.replay()
     torch.cuda.synchronize()
     assert torch.equal(F, want)
+
+
+def test_batch_waits_for_steps_left_on_another_stream(B):
+    """The contexts' streams were changed after the steps were left there; the batch takes their operand copies, state
+    buffers and schedules."""
+    ctxs = [_dense(B, n)[0] for n in (200, 300, 260)]
+    R, n = 16, 260
+    sched = B.make_schedule(c0=1.0, prec=1, readout_every=0)
+    S, Y = _state(R, n, 1)
+    B.veloxq_steps_dev(ctxs[2], R, 0, 3, 20, sched, S, Y)
+    torch.cuda.synchronize()
+    want = (S, Y, B.veloxq_solve_batch(ctxs, R, 20, sched, seed=4))
+    S, Y = _state(R, n, 1)
+    torch.cuda.synchronize()
+    s1 = torch.cuda.Stream()
+    with torch.cuda.stream(s1):
+        torch.cuda._sleep(HOLD)
+        B.veloxq_steps_dev(ctxs[2], R, 0, 3, 20, sched, S, Y)
+        e1 = s1.record_event()
+    # not the default stream, which would wait for every other one
+    s2 = torch.cuda.Stream()
+    for c in ctxs:
+        B.veloxq_set_stream(c, s2.cuda_stream)
+    got = B.veloxq_solve_batch(ctxs, R, 20, sched, seed=4)
+    assert e1.query()
+    assert torch.equal(S, want[0]) and torch.equal(Y, want[1])
+    assert np.array_equal(got["E"], want[2]["E"])
+    assert all(np.array_equal(a, b) for a, b in zip(got["x"], want[2]["x"]))
