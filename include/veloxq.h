@@ -273,7 +273,14 @@ int veloxq_hubo3_reduce_local(int64_t n, const double* h, int64_t n2, const int6
  * Runs on the current device and the default stream. */
 int veloxq_selftest_timeout(int64_t budget_cycles);
 
-/* Release every device and host resource of ctx (NULL is a no-op). */
+/* The same wait as a call on ctx that returns before its kernels end (see
+ * veloxq_steps_dev): runs out on ctx's stream and is reported as such a call's
+ * would be. Returns OK; EINVAL as above or for a NULL ctx. */
+int veloxq_selftest_timeout_async(veloxq_ctx* ctx, int64_t budget_cycles);
+
+/* Release every device and host resource of ctx (NULL is a no-op). A wait
+ * that gave up in a call not yet waited for goes unreported: use
+ * veloxq_synchronize first. */
 void veloxq_destroy(veloxq_ctx* ctx);
 
 /* Thread-local message describing the last non-OK status of this thread. */
@@ -286,6 +293,12 @@ int veloxq_get_info(veloxq_ctx* ctx, veloxq_info* info);
  * a NULL stream runs on a stream the context owns, ordered after the legacy
  * default stream; on a non-NULL stream it runs (and is graph-captured) there. */
 int veloxq_set_stream(veloxq_ctx* ctx, void* stream);
+
+/* Waits for the work that calls on ctx left on its stream, and for kernels that
+ * a call on another stream left on its scratch. Errors: ETIMEDOUT if a bounded
+ * wait gave up in one of them (the results of that call and of those issued
+ * after it are not valid; the next call starts clean), EINVAL in capture. */
+int veloxq_synchronize(veloxq_ctx* ctx);
 
 /* Timing of the last veloxq_solve or veloxq_grad on ctx (EINVAL if none ran yet). */
 int veloxq_last_timing(veloxq_ctx* ctx, veloxq_timing* timing);
@@ -378,7 +391,9 @@ int veloxq_energy_dev_noalloc(veloxq_ctx* ctx, int64_t batch, const uint8_t* X, 
  * Pieces of the step, for parity tests and for callers that drive the
  * integration themselves (device pointers, asynchronous). A bounded wait of
  * the tensor-core kernels that gives up after a call has returned is reported
- * (ETIMEDOUT) by the next call on the context.
+ * (ETIMEDOUT, once) by the next call on the context that finds it, and by
+ * veloxq_synchronize in any case: call that before trusting the results of
+ * the last step or field.
  * ------------------------------------------------------------------------- */
 
 /* Philox initial state S, Y [R][n] for seed and sigma0 (same draw as solve). */

@@ -34,7 +34,7 @@ EXPORTED = [
     "veloxq_solve", "veloxq_solve_batch", "veloxq_energy", "veloxq_energy_dev", "veloxq_init_state_dev",
     "veloxq_field_dev", "veloxq_steps_dev", "veloxq_spectral_radius", "veloxq_grad", "veloxq_last_timing",
     "veloxq_batch_state_dev", "veloxq_energy_dev_noalloc", "veloxq_hubo3_reduce", "veloxq_hubo3_reduce_local",
-    "veloxq_selftest_timeout",
+    "veloxq_selftest_timeout", "veloxq_selftest_timeout_async", "veloxq_synchronize",
 ]
 
 
@@ -97,6 +97,8 @@ def _load():
         "veloxq_hubo3_reduce": (I, [I64, P, I64, P, P, P, I64, P, P, P, P, P, P, P, P, P, P, P]),
         "veloxq_hubo3_reduce_local": (I, [I64, P, I64, P, P, P, I64, P, P, P, P, P, P, P, P, P, P, P, P]),
         "veloxq_selftest_timeout": (I, [I64]),
+        "veloxq_selftest_timeout_async": (I, [P, I64]),
+        "veloxq_synchronize": (I, [P]),
     }
     for name, (res, args) in sig.items():
         fn = getattr(lib, name)
@@ -279,6 +281,17 @@ def veloxq_selftest_timeout(budget_cycles: int) -> None:
     """Run the bounded-wait self-test (raises VeloxqError: ETIMEDOUT is the
     expected outcome)."""
     _check(_lib.veloxq_selftest_timeout(int(budget_cycles)))
+
+
+def veloxq_selftest_timeout_async(ctx: Context, budget_cycles: int) -> None:
+    """The self-test's wait as a call that returns before its kernels end: reported by a later call on ctx."""
+    veloxq_set_stream(ctx, _stream_ptr())
+    _check(_lib.veloxq_selftest_timeout_async(ctx.handle, int(budget_cycles)))
+
+
+def veloxq_synchronize(ctx: Context) -> None:
+    """Wait for the steps and fields left running on ctx and raise if a bounded wait gave up in one of them."""
+    _check(_lib.veloxq_synchronize(ctx.handle))
 
 
 def veloxq_destroy(ctx: Context):

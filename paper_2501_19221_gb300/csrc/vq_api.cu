@@ -940,7 +940,12 @@ int veloxq_solve_batch(veloxq_ctx* const* ctxs, int32_t count, int32_t replicas,
     CtxExtra* ex = extra(c0);
     cudaStream_t st = ex->work;
     for (int32_t m = 0; m < count; ++m) {
-        VQ_TRY(order_behind_pending(ctxs[m], st));   // steps left on another stream than the context's
+        // steps left on another stream than the context's, and a wait that gave up in them
+        VQ_TRY(order_behind_pending(ctxs[m], ctxs[m]->stream));
+        const int earlier = t32_check(ctxs[m]);
+        if (earlier != VELOXQ_OK) return fail(earlier, "instance " + std::to_string(m) + ": " + g_err);
+    }
+    for (int32_t m = 0; m < count; ++m) {
         if (m > 0 && ctxs[m]->stream == ctxs[m - 1]->stream) continue;   // ordered already
         VQ_CUDA(cudaEventRecord(ex->ev, ctxs[m]->stream));
         VQ_CUDA(cudaStreamWaitEvent(st, ex->ev, 0));
@@ -1225,6 +1230,30 @@ int veloxq_steps_dev(veloxq_ctx* ctx, int32_t R, int32_t k_begin, int32_t k_coun
     VQ_TRY(launch_transpose(ctx->stream, ctx->y.as<float>(), Y, n, R));
     if (F_last) VQ_TRY(launch_transpose(ctx->stream, ctx->f.as<float>(), F_last, n, R));
     return VELOXQ_OK;
+}
+
+int veloxq_synchronize(veloxq_ctx* ctx) {
+    if (!ctx) return fail(VELOXQ_EINVAL, "ctx must not be NULL");
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    VQ_CUDA(cudaStreamIsCapturing(ctx->stream, &cs));
+    if (cs != cudaStreamCaptureStatusNone) return fail(VELOXQ_EINVAL, "the context's stream is in capture");
+    VQ_CUDA(cudaStreamSynchronize(ctx->stream));
+    CtxExtra* ex = extra(ctx);
+    if (ex && ex->apending) {
+        VQ_CUDA(cudaEventSynchronize(ex->aev));
+        ex->apending = false;
+    }
+    return check_device(ctx);
+}
+
+int veloxq_selftest_timeout_async(veloxq_ctx* ctx, int64_t budget_cycles) {
+    if (!ctx) return fail(VELOXQ_EINVAL, "ctx must not be NULL");
+    VQ_TRY(check_device(ctx));
+    if (budget_cycles < 1000 || budget_cycles > 10000000000LL)
+        return fail(VELOXQ_EINVAL, "budget_cycles must be in [1e3, 1e10]");
+    EarlyReturn early{ctx};
+    VQ_TRY(async_words(ctx));
+    return tc_wait_selftest_async(ctx, (long long)budget_cycles);
 }
 
 int veloxq_selftest_timeout(int64_t budget_cycles) {

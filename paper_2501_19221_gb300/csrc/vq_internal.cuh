@@ -287,6 +287,7 @@ int tc_maps(veloxq_ctx* ctx, int prec, int terms, int32_t R, void* sop0, void* s
             CUtensorMap* ms0, CUtensorMap* ms1, CUtensorMap* ms0_lo, CUtensorMap* ms1_lo);
 int tc_quant_s(veloxq_ctx* ctx, int prec, int32_t R, const float* S, void* sop, const Rule& rule = Rule());
 size_t tc_sop_bytes(veloxq_ctx* ctx, int prec, int terms, int32_t R);
+int tc_wait_selftest_async(veloxq_ctx* ctx, long long budget);
 int tc_wait_selftest(long long budget, int* code_out);   // the bounded wait run out on purpose
 // Steps k_begin .. k_end - 1 in one launch (tiles of consecutive steps
 // overlap, each waiting only for the column block of the state it reads).
@@ -312,6 +313,7 @@ struct T32Run {
     int terms = 3;        // BF16 terms of the operand
     uint32_t seq = 0;     // sequence number of its range check (0: not checked)
 };
+int check_device(veloxq_ctx* ctx);  // current device, order behind calls on other streams, their late errors
 int async_words(veloxq_ctx* ctx);   // allocates and zeroes t32w and t32h (once)
 int t32_prepare(veloxq_ctx* ctx, int32_t R, bool* ready);
 int t32_split(veloxq_ctx* ctx, int32_t R, const float* S, const Rule& rule, bool check, T32Run* t);

@@ -92,6 +92,8 @@ extern "C" int veloxq_energy_dev_noalloc(veloxq_ctx* ctx, int64_t batch, const u
     int dev = -1;
     VQ_CUDA(cudaGetDevice(&dev));
     if (dev != ctx->device) return fail(VELOXQ_EINVAL, "the context's device must be the current device");
+    // a wait that gave up in an earlier call (a word of host memory)
+    if (ctx->t32h.p && *static_cast<volatile int*>(ctx->t32h.p)) VQ_TRY(check_device(ctx));
     const int64_t groups = ctx->dense ? div_up(ctx->n, 64) : 64;   // partial sums per vector
     if (batch > 65535 || batch * groups > kNoAllocParts)
         return fail(VELOXQ_EINVAL, "batch too large for the fixed scratch of veloxq_energy_dev_noalloc: need batch <= " +

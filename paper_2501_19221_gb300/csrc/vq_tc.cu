@@ -424,7 +424,7 @@ __global__ void __launch_bounds__(320, 1) k_tc_step(const __grid_constant__ CUte
 // The bounded wait of the kernels above on a barrier that nothing arrives on:
 // it runs out after `budget` cycles, records its code in the error word and
 // returns (the path every kernel takes when a wait gives up).
-__global__ void k_wait_selftest(int* err, long long budget) {
+__global__ void k_wait_selftest(int* err, long long budget, int* err_host) {
     __shared__ __align__(8) uint64_t bar;
     if (threadIdx.x == 0) {
         mbar_init(&bar, 1);
@@ -433,6 +433,10 @@ __global__ void k_wait_selftest(int* err, long long budget) {
     __syncthreads();
     if (threadIdx.x == 0) mbar_wait(&bar, 0, err, TC_ERR_SELFTEST, budget);
     __syncthreads();
+    if (threadIdx.x == 0 && err_host) {
+        const int e = *(volatile int*)err;
+        if (e) atomicOr_system(err_host, e);
+    }
 }
 
 // ---- operand preparation --------------------------------------------------
@@ -637,13 +641,20 @@ int tc_wait_selftest(long long budget, int* code_out) {
     int h = 0;
     cudaError_t e = cudaMemset(err, 0, sizeof(int));
     if (e == cudaSuccess) {
-        k_wait_selftest<<<1, 32>>>(err, budget);
+        k_wait_selftest<<<1, 32>>>(err, budget, nullptr);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaMemcpy(&h, err, sizeof(int), cudaMemcpyDeviceToHost);
     cudaFree(err);
     if (e != cudaSuccess) return cuda_fail(e, "wait self-test");
     *code_out = h;
+    return VELOXQ_OK;
+}
+
+// The same as a call that returns early does it: on the context's stream, with its error words.
+int tc_wait_selftest_async(veloxq_ctx* ctx, long long budget) {
+    k_wait_selftest<<<1, 32, 0, ctx->stream>>>(ctx->t32w.as<int>(), budget, static_cast<int*>(ctx->t32h.dev));
+    VQ_LAUNCH_CHECK("wait self-test");
     return VELOXQ_OK;
 }
 

@@ -861,17 +861,23 @@ int t32_run(veloxq_ctx* ctx, int32_t R, T32Run* t, float** cur, float** nxt, flo
     return VELOXQ_OK;
 }
 
-// Whether a wait of an earlier call on ctx gave up (reported once).
+// Whether a wait of an earlier call on ctx gave up (reported once, and to a
+// call in capture without ending the report, which takes a synchronisation).
 int t32_check(veloxq_ctx* ctx) {
     if (!ctx->t32h.p) return VELOXQ_OK;
     volatile int* h = static_cast<volatile int*>(ctx->t32h.p);
     const int code = h[0];
     if (!code) return VELOXQ_OK;
-    VQ_CUDA(cudaStreamSynchronize(ctx->stream));
-    h[0] = 0;
-    VQ_CUDA(cudaMemsetAsync(ctx->t32w.p, 0, sizeof(int), ctx->stream));
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    VQ_CUDA(cudaStreamIsCapturing(ctx->stream, &cs));
+    if (cs == cudaStreamCaptureStatusNone) {
+        VQ_CUDA(cudaStreamSynchronize(ctx->stream));
+        h[0] = 0;
+        VQ_CUDA(cudaMemsetAsync(ctx->t32w.p, 0, sizeof(int), ctx->stream));
+    }
     return fail(VELOXQ_ETIMEDOUT, "a bounded device wait in an earlier call on this context gave up (code " +
-                                      std::to_string(code) + "); its results are not valid");
+                                      std::to_string(code) + "); its results, and those of the calls issued since, "
+                                      "are not valid");
 }
 
 }  // namespace vq
