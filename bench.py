@@ -583,11 +583,11 @@ def tc_roofline(prec, method, n, R, per_ms):
 
 def fp32_roofline(n, R, method, per_ms):
     """Roofline of one FP32-accurate step on the tensor cores (k_t32, and
-    k_t32_finish when the k-loop is split): six BF16 products of 2 n^2 R FLOP
+    k_t32_finish when the k-loop is split): eight BF16 products of 2 n^2 R FLOP
     (three for Parallel Annealing, whose operand is one exact term) against
     the measured BF16 peak."""
     peaks, src = _peaks()
-    terms = 3 if method == "pa" else 6
+    terms = 3 if method == "pa" else 8
     flops = 2.0 * n * n * R * terms
     ach = flops / (per_ms / 1e3) / 1e12
     return {"kernel": "k_t32", "bound": "tensor", "achieved": ach, "peak": peaks["bf16_tflops"], "unit": "TFLOP/s",
@@ -634,7 +634,7 @@ def time_to_target(B, stream, seeds=32, n=8192, R=1024, K=200, method=0):
     construction); a form reaches it at the smallest K' of TTT_GRID where at
     least half of the seeds end at or below E*. Times are CUDA-event times of
     whole solves (median over the seeds). The FP32 form's step is also given
-    as its own roofline fraction (its six BF16 products, three for Parallel
+    as its own roofline fraction (its eight BF16 products, three for Parallel
     Annealing, against the BF16 peak), so that the ratios can be read against
     the quality of the baseline kernel."""
     import torch

@@ -71,9 +71,10 @@ typedef enum { VELOXQ_I8 = 0, VELOXQ_I32 = 1, VELOXQ_F32 = 2, VELOXQ_F64 = 3 } v
 /* Operand precision of the dense local-field product F = Qoff S. All run on
  * the tcgen05 tensor cores and accumulate in FP32. Sparse contexts always use
  * FP32 (or exact int8 couplings).
- *   FP32:          every operand as the exact sum of three BF16 terms, the six
- *                  term products down to 2^-16 of the leading one (error
- *                  against FP64 below that of an FP32 sum of products); small
+ *   FP32:          every operand as the exact sum of three BF16 terms, eight
+ *                  of their nine products (error against FP64 that of an FP32
+ *                  sum of products on rows of one coupling, below it on longer
+ *                  ones); small
  *                  n, and values whose terms would leave BF16's range (not
  *                  finite, |x| >= 2^127, 0 < |x| < 2^-100), as FP32 sums of
  *                  products on the CUDA cores.

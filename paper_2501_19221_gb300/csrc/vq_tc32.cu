@@ -4,26 +4,38 @@
 //
 // Every FP32 operand is written as the exact sum of three BF16 terms
 // (x = x1 + x2 + x3: 6, 8 and up to 9 significant bits), and the product is the
-// sum of the six term products down to 2^-16 of the leading one,
-//     q s ~ q1 s1 + (q1 s2 + q2 s1) + (q2 s2 + q1 s3 + q3 s1);
-// the three that are left out are below 2^-22 of q s. For Parallel Annealing
-// the operand is +-1, one exact term, and three products are the whole of q s.
+// sum of eight of the nine term products,
+//     q s ~ q1 s1 + (q1 s2 + q2 s1) + (q2 s2 + q1 s3 + q3 s1) + (q2 s3 + q3 s2);
+// the one that is left out, q3 s3, is below 2^-29 of q s (x2 is at most 2^-6
+// of x, x3 at most 2^-14). The last two reach 2^-20 of q s together: without
+// them a row of one coupling had 3.4 times the error of an FP32 product, one
+// of six twice that of an FP32 sum, and rows of fewer than about 100
+// couplings were less exact than such a sum. For Parallel Annealing the
+// operand is +-1, one exact term, and three products are the whole of q s.
 //
 // Accuracy: the products of BF16 terms are exact in FP32, but the tensor
 // cores' accumulation cuts its sums off toward zero, a relative shrinking that
-// adds up over the steps of a run. Three things keep it small: the leading
+// adds up over the steps of a run. Four things keep it small: the leading
 // term has 6 bits only, so that a sum of leading products is mostly exact in
 // 24 bits (with 8-bit leading terms the field shrank by 5.8e-8, with 6 bits by
-// 3e-9 at 32 variables); the five small products go to an accumulator of their
-// own (sharing one: 8.3e-8); and both are drained after every 64 or 128
-// variables into FP32 registers with rounded additions. Error against FP64
-// (normwise, N(0, 1/n) couplings, S uniform in [-1, 1]), the FP32 SGEMM of
-// vq_dense.cu -> here: n = 600: 2.2e-7 -> 1.0e-7, 2048: 2.2e-7 -> 1.1e-7,
-// 4096: 5.1e-7 -> 1.2e-7, 8192: 1.6e-6 -> 1.7e-7.
+// 3e-9 at 32 variables); the seven small products go to an accumulator of their
+// own (sharing one: 8.3e-8); both are drained after every 64 or 128
+// variables into FP32 registers with rounded additions; and the two parts
+// stay apart in these until the last drain, so that few couplings, whose
+// leading sums are exact, are rounded once. Error against FP64 (normwise, S
+// uniform in [-1, 1]), the FP32 SGEMM of vq_dense.cu -> here, N(0, 1/n)
+// couplings: n = 600: 2.2e-7 -> 6.0e-8, 2048: 3.1e-7 -> 7.0e-8, 4096:
+// 5.8e-7 -> 9.2e-8, 8192: 1.6e-6 -> 1.6e-7. Rows of few couplings, n = 700 /
+// 2600: one 2.6e-8 -> 2.6e-8 / the same, two 3.6e-8 -> 3.5e-8 / 3.5e-8 ->
+// 2.5e-8, six 5.0e-8 -> 4.5e-8 / 4.8e-8 -> 2.5e-8, 64 8.1e-8 -> 5.0e-8 /
+// 9.2e-8 -> 3.1e-8. Log-normal couplings (sigma 3): 2.0e-7 -> 1.4e-7 / 4.7e-7
+// -> 2.1e-7. States of about four variables on full rows: 4.5e-8 -> 4.1e-8 /
+// 4.4e-8 -> 2.5e-8.
 //
-// Time per step, SGEMM -> here: n = 8192, R = 1024: 4060 -> 580 us (0.74 of
-// the measured BF16 rate at 12 n^2 R FLOP); n = 8192, R = 64: 650 -> 100 us;
-// n = 3000, R = 1000: 690 -> 130 us; n = 1001, R = 100: 41 -> 13 us.
+// Time per step, SGEMM -> here: n = 8192, R = 1024: 4060 -> 625 us (0.92 of
+// the measured BF16 rate at 16 n^2 R FLOP; with six products 548); n = 8192,
+// R = 64: 650 -> 100 us; n = 3000, R = 1000: 690 -> 99 us; n = 1001, R = 100:
+// 41 -> 11.8 us.
 //
 // CTA pairs (clusters of 2, cta_group::2) compute 256 x 128 tiles (rows x
 // replicas), M = 256 MMAs issued by the even CTA, operands staged by TMA in
@@ -40,7 +52,7 @@
 //     The two launches of a step follow each other by programmatic dependent
 //     launch. The choice depends on n and R alone, so a run gives the same
 //     bits however it is cut into calls.
-// What bounds it: the tensor cores at large n (12 n^2 R FLOP per step);
+// What bounds it: the tensor cores at large n (16 n^2 R FLOP per step);
 // with few replicas the 6 bytes per coupling of the three term planes.
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -129,26 +141,14 @@ __device__ __forceinline__ void tma_load_3d_pair(void* dst, const CUtensorMap* m
         ::"r"(smem_u32(dst)), "l"((uint64_t)map), "r"(x), "r"(y), "r"(0), "r"(bar_cl)
         : "memory");
 }
-// 32 columns of each of two accumulators
-__device__ __forceinline__ void tmem_ld32x2(uint32_t ta, uint32_t tb, uint32_t (&v)[32], uint32_t (&w)[32]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
-          "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
-          "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-        : "r"(ta));
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-        : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7]),
-          "=r"(w[8]), "=r"(w[9]), "=r"(w[10]), "=r"(w[11]), "=r"(w[12]), "=r"(w[13]), "=r"(w[14]), "=r"(w[15]),
-          "=r"(w[16]), "=r"(w[17]), "=r"(w[18]), "=r"(w[19]), "=r"(w[20]), "=r"(w[21]), "=r"(w[22]), "=r"(w[23]),
-          "=r"(w[24]), "=r"(w[25]), "=r"(w[26]), "=r"(w[27]), "=r"(w[28]), "=r"(w[29]), "=r"(w[30]), "=r"(w[31])
-        : "r"(tb));
+// 8 columns of each of two accumulators
+__device__ __forceinline__ void tmem_ld8x2(uint32_t ta, uint32_t tb, uint32_t (&v)[8], uint32_t (&w)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+                 : "r"(ta));
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
+                 : "r"(tb));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
@@ -296,7 +296,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_t32(const __grid_constant__ CUte
                         if constexpr (NB == 3) {
                             const uint64_t b1 = desc128(sb + B_TERM + o), b2 = desc128(sb + 2 * B_TERM + o);
                             mma_pair<BN>(d, a0, b0, acc);
-                            mma_pair<BN>(dx, a0, b2, acc);
+                            mma_pair<BN>(dx, a1, b2, acc);
+                            mma_pair<BN>(dx, a2, b1, 1u);
+                            mma_pair<BN>(dx, a0, b2, 1u);
                             mma_pair<BN>(dx, a0, b1, 1u);
                             mma_pair<BN>(dx, a1, b1, 1u);
                             mma_pair<BN>(dx, a1, b0, 1u);
@@ -328,26 +330,30 @@ __global__ void __launch_bounds__(THREADS, 1) k_t32(const __grid_constant__ CUte
         for (int64_t g = pair; g < work && ok; g += pairs) {
             int j, r, c, kb0, kb1;
             item(g, j, r, c, kb0, kb1);
-            float F[NC];
+            float F[NC], L[NC];
 #pragma unroll
-            for (int v = 0; v < NC; ++v) F[v] = 0.0f;
+            for (int v = 0; v < NC; ++v) F[v] = L[v] = 0.0f;
             for (int kb = kb0; kb < kb1; kb += a.drain, ++it) {
                 const uint32_t b = it & 1u;
                 if (!mbar_wait<true>(&accf[b], (it >> 1) & 1u, a.err, TC_ERR_EPILOGUE)) { ok = false; break; }
                 tc_fence_after();
 #pragma unroll
-                for (int h = 0; h < NC / 32; ++h) {
-                    uint32_t v[32], x[32];
-                    tmem_ld32x2(tcol + b * 2 * BN + h * 32, tcol + b * 2 * BN + BN + h * 32, v, x);
+                for (int h = 0; h < NC / 8; ++h) {
+                    uint32_t v[8], x[8];
+                    tmem_ld8x2(tcol + b * 2 * BN + h * 8, tcol + b * 2 * BN + BN + h * 8, v, x);
 #pragma unroll
-                    for (int l = 0; l < 32; ++l)
-                        F[h * 32 + l] = __fadd_rn(F[h * 32 + l], __fadd_rn(__uint_as_float(v[l]), __uint_as_float(x[l])));
+                    for (int l = 0; l < 8; ++l) {
+                        F[h * 8 + l] = __fadd_rn(F[h * 8 + l], __uint_as_float(v[l]));
+                        L[h * 8 + l] = __fadd_rn(L[h * 8 + l], __uint_as_float(x[l]));
+                    }
                 }
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive_remote(acce_cl + b * 8);
             }
             if (!ok) break;
+#pragma unroll
+            for (int v = 0; v < NC; ++v) F[v] = __fadd_rn(F[v], L[v]);
             const int row = r * (2 * BM) + (int)rank * BM + q * 32 + lane;
             const int r0 = c * BN + half * NC;
             const bool row_ok = row < a.n;
@@ -804,8 +810,8 @@ int t32_run(veloxq_ctx* ctx, int32_t R, T32Run* t, float** cur, float** nxt, flo
     a.kper = p.kper;
     a.ksplit = p.ksplit;
     // Tensor-core accumulation cuts its sums off toward zero, so F shrinks by a part that grows with the variables
-    // between two drains: 3e-9 at 32, 7e-9 at 64, 1.8e-8 at 128. It is kept below about 3 % of the error the FP32
-    // SGEMM has at that size (2e-7 up to n = 2048, 5e-7 at 4096, 1.6e-6 at 8192).
+    // between two drains: 3e-9 at 32, 7e-9 at 64, 1.9e-8 at 128. It is kept below about 3 % of the error the FP32
+    // SGEMM has at that size (2e-7 to 3e-7 up to n = 2048, 6e-7 at 4096, 1.6e-6 at 8192).
     // (Parallel Annealing's products with +-1 have 6 and 8 bits and lose nothing at 256.)
     a.drain = terms == 1 ? 4 : n < 2560 ? 1 : 2;
     a.err = ctx->t32w.as<int>();
