@@ -45,7 +45,8 @@
 // replicas rather than 256 keep a thread's part of the drained field in 64
 // registers, and give twice the tiles to spread over the SMs.
 //   * Enough tiles (more than half of the pairs): one launch runs every step
-//     up to a readout, tiles of consecutive steps overlapping as in vq_tc.cu.
+//     up to a readout, tiles of consecutive steps overlapping as in vq_tc.cu
+//     (and one behind it that only works where SMs were held by others).
 //   * Fewer: the k-loop is split over the idle pairs (at least two blocks each; with one, 14 against 13 us per
 //     step at n = 1001, R = 100), the partial fields go to a workspace, and
 //     k_t32_finish adds them in order, updates, and writes the next operand.
@@ -172,10 +173,45 @@ struct T32Args {
     int32_t drain;               // k-blocks accumulated in tensor memory between two drains
     int* err;                    // device error word of the bounded waits
     int* err_host;               // the same, in mapped host memory
-    uint32_t* done;              // [replica column blocks] finished epilogue warps (zeroed per launch)
+    uint32_t* done;              // [replica column blocks] finished epilogue warps, then the lists of the pairs that take
+                                 // part in the run and in its shared form (zeroed per run; null for one step)
     const uint32_t* skip;        // do nothing if *skip == skip_seq (null: always run)
     uint32_t skip_seq;
 };
+
+// Which pairs take part in a run of several steps. Tiles wait for those of
+// the step before, so every pair that owns tiles has to be resident; another
+// kernel may hold SMs for longer than a wait lasts. Pairs therefore put
+// themselves on a list (its count in the low 16 bits) before they begin. Where
+// all of the grid are there, the tiles go to the pairs by their place in the
+// grid. Where one has waited `patience` cycles it closes the list (top bit, the
+// count so far in bits 16 to 30), all leave without having done anything, and
+// the launch behind this one (SHARED, which leaves at once in the ordinary
+// case) makes a list of its own and deals the tiles to the pairs on it. Which
+// pair computes a tile does not change a bit. Two launches, because a kernel
+// that takes its share of the tiles from a list at run time is 7 % slower (676
+// against 630 us per step at n = 8192, R = 1024).
+// Returns this pair's number on the list and the pairs that take part (0: it came too late).
+constexpr uint32_t LIST_CLOSED = 0x80000000u;
+constexpr long long kListPatience = kWaitCycles / 4, kListPatienceShared = kWaitCycles / 1000;   // ~0.5 s, ~2 ms
+__device__ __forceinline__ void join_list(uint32_t* list, uint32_t grid_pairs, long long patience, uint32_t& me,
+                                          uint32_t& pairs) {
+    me = atomicAdd(list, 1u);
+    pairs = 0;
+    if (me & LIST_CLOSED) {
+        me = 0;
+        return;
+    }
+    const long long t0 = clock64();
+    while (true) {
+        const uint32_t w = ld_acquire_u32(list);
+        if ((w & LIST_CLOSED) || w == grid_pairs) {
+            pairs = w & LIST_CLOSED ? (w >> 16) & 0x7fffu : w;
+            return;
+        }
+        if (clock64() - t0 > patience) atomicCAS(list, w, w | LIST_CLOSED | (w << 16));
+    }
+}
 
 // form of the kernel: what the epilogue does with the field
 enum { FORM_BSB = 0, FORM_ASB = 1, FORM_PA = 2, FORM_FIELD = 3, FORM_SPLIT = 4 };
@@ -184,9 +220,9 @@ enum { FORM_BSB = 0, FORM_ASB = 1, FORM_PA = 2, FORM_FIELD = 3, FORM_SPLIT = 4 }
 // step's field per work item). Tile order and the dependency counters between
 // steps are those of k_tc_step (vq_tc.cu): tile g = j * tiles + t of step
 // k + j starts only after every epilogue warp of its replica column block has
-// finished step j - 1, a pair only waits for tiles with a lower g, all CTAs
-// are resident, and every wait is bounded.
-template <int NB, int FORM, int BN = BN_WIDE>
+// finished step j - 1, a pair only waits for tiles with a lower g, all pairs
+// that own tiles are resident (join_list), and every wait is bounded.
+template <int NB, int FORM, int BN = BN_WIDE, bool SHARED = false>
 __global__ void __launch_bounds__(THREADS, 1) k_t32(const __grid_constant__ CUtensorMap tmA,
                                                     const __grid_constant__ CUtensorMap tmB0,
                                                     const __grid_constant__ CUtensorMap tmB1, const T32Args a) {
@@ -200,11 +236,12 @@ __global__ void __launch_bounds__(THREADS, 1) k_t32(const __grid_constant__ CUte
     uint64_t* accf = empty + STAGES;      // [2] both CTAs: accumulator buffer holds a block's products
     uint64_t* acce = accf + 2;            // [2] even CTA: buffer drained by both CTAs' epilogues
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acce + 2);
+    uint32_t* listed = tmem_slot + 2;     // [2], 8-byte aligned: this pair's number, the pairs that take part
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_rank();
     const bool leader = rank == 0;
-    const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
+    int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
     const int num_kb = (a.n_pad + BK - 1) / BK;
     const int MT = (a.n + 2 * BM - 1) / (2 * BM), NT = (a.R + BN - 1) / BN;
     const int tiles = MT * NT;
@@ -232,7 +269,36 @@ __global__ void __launch_bounds__(THREADS, 1) k_t32(const __grid_constant__ CUte
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const bool skip = a.skip && *a.skip == a.skip_seq;
-    const int64_t work = skip ? 0 : FORM == FORM_SPLIT ? (int64_t)tiles * a.ksplit : (int64_t)steps * tiles;
+    if constexpr (SHARED) {
+        if (leader && threadIdx.x == 0) {
+            uint32_t me = 0, all = 0;
+            if (ld_acquire_u32(a.done + NT) & LIST_CLOSED)
+                join_list(a.done + NT + 1, gridDim.x >> 1, kListPatienceShared, me, all);
+            asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(smem_u32(listed)), "r"(me), "r"(all) : "memory");
+            asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(mapa(smem_u32(listed), 1)), "r"(me), "r"(all)
+                         : "memory");
+        }
+        __syncwarp();
+        cluster_sync();
+        pair = (int)*(volatile uint32_t*)listed;
+        pairs = (int)*(volatile uint32_t*)(listed + 1);
+    } else if (a.done) {
+        if (leader && threadIdx.x == 0) {
+            uint32_t me, all;
+            join_list(a.done + NT, gridDim.x >> 1, kListPatience, me, all);
+        }
+        __syncwarp();
+        cluster_sync();
+        if (ld_acquire_u32(a.done + NT) & LIST_CLOSED) {       // final by now: closed, or all are there
+            tc_fence_before();
+            __syncthreads();
+            cluster_sync();
+            tc_fence_after();
+            if (warp == 1) tmem_dealloc(tmem, 4 * BN);
+            return;
+        }
+    }
+    const int64_t work = skip || (SHARED && pairs == 0) ? 0 : FORM == FORM_SPLIT ? (int64_t)tiles * a.ksplit : (int64_t)steps * tiles;
     // work item g: step j, row block r, column block c, k-blocks [kb0, kb1)
     auto item = [&](int64_t g, int& j, int& r, int& c, int& kb0, int& kb1) {
         const int z = (int)(g / tiles), t = (int)(g - (int64_t)z * tiles);
@@ -547,11 +613,11 @@ T32Kernel pick_split(bool exact_operand, int bn) {
         return exact_operand ? k_t32<1, FORM_SPLIT, BN_NARROW> : k_t32<3, FORM_SPLIT, BN_NARROW>;
     return exact_operand ? k_t32<1, FORM_SPLIT> : k_t32<3, FORM_SPLIT>;
 }
-T32Kernel pick(int form) {
+template <bool SHARED> T32Kernel pick(int form) {
     switch (form) {
-        case FORM_BSB: return k_t32<3, FORM_BSB>;
-        case FORM_ASB: return k_t32<3, FORM_ASB>;
-        case FORM_PA: return k_t32<1, FORM_PA>;
+        case FORM_BSB: return k_t32<3, FORM_BSB, BN_WIDE, SHARED>;
+        case FORM_ASB: return k_t32<3, FORM_ASB, BN_WIDE, SHARED>;
+        case FORM_PA: return k_t32<1, FORM_PA, BN_WIDE, SHARED>;
         default: return k_t32<3, FORM_FIELD>;
     }
 }
@@ -686,7 +752,7 @@ int t32_prepare(veloxq_ctx* ctx, int32_t R, bool* ready) {
     if (div_up(n, 256) * (int64_t)R > INT32_MAX || p.tiles > INT32_MAX / 2) return VELOXQ_OK;
     const size_t ob = sizeof(__nv_bfloat16) * 3 * (size_t)R * (size_t)np;
     const size_t pb = p.ksplit > 1 ? sizeof(float) * (size_t)p.ksplit * (size_t)R * (size_t)n : 0;
-    const size_t db = sizeof(uint32_t) * (size_t)p.NT;
+    const size_t db = sizeof(uint32_t) * (size_t)(p.NT + 2);
     const bool fused = p.ksplit == 1;
     if (ctx->q3_state > 0 && ctx->s3[0].bytes >= ob && (!fused || ctx->s3[1].bytes >= ob) && ctx->dpart.bytes >= pb &&
         ctx->tcdone.bytes >= db) {
@@ -771,7 +837,9 @@ bool t32_bad(const veloxq_ctx* ctx, const T32Run& t) {
 
 // launches of `steps` steps up to a readout
 int t32_launches(const veloxq_ctx* ctx, int32_t R, int steps) {
-    return plan(ctx, R).ksplit > 1 ? 2 * steps : (int)div_up(steps, kMaxRunSteps);
+    if (plan(ctx, R).ksplit > 1) return 2 * steps;
+    const int runs = (int)div_up(steps, kMaxRunSteps);
+    return 2 * runs - (steps % kMaxRunSteps == 1 ? 1 : 0);       // a run of more than one step takes two
 }
 
 // Steps k_begin .. k_end - 1 from the operand t32_split (or the last call)
@@ -843,8 +911,9 @@ int t32_run(veloxq_ctx* ctx, int32_t R, T32Run* t, float** cur, float** nxt, flo
             a.group = G;
             break;
         }
-    T32Kernel fn = pick(form);
-    VQ_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T32_SMEM));
+    T32Kernel fn = pick<false>(form), fn_shared = pick<true>(form);
+    for (T32Kernel f : {fn, fn_shared})
+        VQ_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T32_SMEM));
     for (int k0 = k_begin; k0 < k_end; k0 += kMaxRunSteps) {
         const int k1 = std::min(k_end, k0 + kMaxRunSteps), steps = k1 - k0;
         a.k = k0;
@@ -855,10 +924,11 @@ int t32_run(veloxq_ctx* ctx, int32_t R, T32Run* t, float** cur, float** nxt, flo
         a.F_out = k1 == k_end ? F_out : nullptr;
         a.done = nullptr;
         if (steps > 1) {
-            VQ_CUDA(cudaMemsetAsync(ctx->tcdone.p, 0, sizeof(uint32_t) * (size_t)p.NT, ctx->stream));
+            VQ_CUDA(cudaMemsetAsync(ctx->tcdone.p, 0, sizeof(uint32_t) * (size_t)(p.NT + 2), ctx->stream));
             a.done = ctx->tcdone.as<uint32_t>();
         }
         VQ_TRY(launch(ctx, fn, std::min<int64_t>(p.tiles * steps, p.pairs), mq, ms, a));
+        if (steps > 1) VQ_TRY(launch(ctx, fn_shared, std::min<int64_t>(p.tiles * steps, p.pairs), mq, ms, a));
         if ((steps & 1) && !field_only) {
             std::swap(*cur, *nxt);
             t->cur ^= 1;
