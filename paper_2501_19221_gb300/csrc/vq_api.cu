@@ -781,7 +781,8 @@ int veloxq_solve(veloxq_ctx* ctx, int32_t replicas, int32_t steps, const veloxq_
         T32Run t32r;
         bool use_t32 = false;
         if (path == VELOXQ_PATH_DENSE && !use_tc && !dense_ordered(ctx, p, path)) {
-            if (p.sigma0 == 0.0f || p.sigma0 >= 6.6174449e-24f /* 2^-77: |s| >= 2^-100 or 0 */)
+            // 2^-77: |s| >= 2^-100 or 0; 2^120: well below 2^127, where a value may round past BF16's largest
+            if (p.sigma0 == 0.0f || (p.sigma0 >= 6.6174449e-24f && p.sigma0 <= 1.329228e36f))
                 VQ_TRY(t32_prepare(ctx, replicas, &use_t32));
             if (!use_t32) VQ_TRY(dense_prepare(ctx, replicas));
         }
