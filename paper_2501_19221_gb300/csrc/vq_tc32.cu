@@ -93,7 +93,9 @@ __device__ __forceinline__ void split3(float x, __nv_bfloat16 (&t)[3]) {
         t[1] = t[2] = __float2bfloat16_rn(0.0f);
         return;
     }
-    const float a = __uint_as_float((u + 0x0001ffffu + ((u >> 18) & 1u)) & 0xfffc0000u);
+    // (cut instead of rounded from 2^127 on, where rounding may reach infinity; adiabatic SB's states have no bound)
+    const uint32_t up = (u & 0x7f800000u) < (254u << 23) ? 0x0001ffffu + ((u >> 18) & 1u) : 0u;
+    const float a = __uint_as_float((u + up) & 0xfffc0000u);
     const float r = __fsub_rn(x, a);
     t[0] = __float2bfloat16_rn(a);
     t[1] = __float2bfloat16_rn(r);
@@ -419,7 +421,12 @@ __global__ void __launch_bounds__(THREADS, 1) k_t32(const __grid_constant__ CUte
             }
             if (!ok) break;
 #pragma unroll
-            for (int v = 0; v < NC; ++v) F[v] = __fadd_rn(F[v], L[v]);
+            for (int v = 0; v < NC; ++v) {
+                // An infinite state is its own first term: the leading products are then the whole of F, and the small
+                // ones may be infinite with the other sign, or 0 times infinity.
+                const float t = __fadd_rn(F[v], L[v]);
+                F[v] = fabsf(F[v]) == __int_as_float(0x7f800000) ? F[v] : t;
+            }
             const int row = r * (2 * BM) + (int)rank * BM + q * 32 + lane;
             const int r0 = c * BN + half * NC;
             const bool row_ok = row < a.n;

@@ -34,3 +34,31 @@ def test_largest_start_states(B, n, R):
     assert bool(torch.isfinite(S).all())
     X = (S > 0).to(torch.uint8).cpu().numpy()
     assert np.array_equal(got["E_per_replica"], B.veloxq_energy(ctx, X)["E"])
+
+
+@pytest.mark.parametrize("n,R", [(700, 20), (2600, 520)])
+def test_state_that_overflows_within_a_call(B, n, R):
+    """Adiabatic SB has no walls: variable 11 of replica 3 starts at 1e12 and is infinite after two steps. The field of
+    the third step is that of the FP32 sums of products (which a replica outside the terms' range selects): infinite
+    with the coupling's sign, undefined for the variable itself, and the other replicas are not touched."""
+    J, _ = I.sk_qubo(n, seed=0)
+    ctx = B.veloxq_create_ising_dense(J)
+    sched = B.make_schedule(c0=1.0, method=1)
+    g = torch.Generator(device="cuda").manual_seed(1)
+    S = torch.rand(R + 1, n, generator=g, device="cuda") * 0.2 - 0.1
+    S[3, 11] = 1e12
+    S[R, 5] = 1e-36
+    out = []
+    for r in (R, R + 1):
+        s, y = S[:r].clone(), torch.zeros(r, n, device="cuda")
+        f = torch.empty_like(s)
+        B.veloxq_steps_dev(ctx, r, 0, 3, 20, sched, s, y, f)
+        torch.cuda.synchronize()
+        out.append(f[:R])
+    a, b = out
+    other = torch.arange(n, device="cuda") != 11
+    assert bool(torch.isinf(b[3, other]).all())
+    assert torch.equal(a[3, other], b[3, other]) and bool(torch.isnan(a[3, 11])) and bool(torch.isnan(b[3, 11]))
+    keep = torch.arange(R, device="cuda") != 3
+    assert bool(torch.isfinite(a[keep]).all())
+    assert float((a[keep] - b[keep]).norm() / b[keep].norm()) <= 1e-5
