@@ -77,7 +77,12 @@ typedef enum { VELOXQ_I8 = 0, VELOXQ_I32 = 1, VELOXQ_F32 = 2, VELOXQ_F64 = 3 } v
  *                  ones); small
  *                  n, and values whose terms would leave BF16's range (not
  *                  finite, |x| >= 2^127, 0 < |x| < 2^-100), as FP32 sums of
- *                  products on the CUDA cores.
+ *                  products on the CUDA cores. The terms of Qoff (6 n^2 bytes)
+ *                  stay with the context from the first such call; a call for
+ *                  which they and the state's terms (up to 12 R n bytes) find
+ *                  no room, or for which they would take more than half of the
+ *                  memory that is free, runs as FP32 sums too (other roundings,
+ *                  so other bits).
  *   BF16:          bf16(Qoff) x bf16(s).
  *   FP8:           Qoff as E4M3 with one FP32 scale per row (amax_i / 448);
  *                  S (whose entries the walls keep in [-1, 1]) with the fixed

@@ -749,7 +749,7 @@ int async_words(veloxq_ctx* ctx) {
 // Prepares the form for R replicas: the term planes of Qoff (once per
 // context), operand and counter buffers. *ready = false (and no error) where
 // the SGEMM has to serve: small n, values whose terms leave BF16's range, or
-// no room for the planes. Allocates; with the stream in capture, *ready tells
+// no room (for this call: the next one tries again). Allocates; with the stream in capture, *ready tells
 // whether everything was there already.
 int t32_prepare(veloxq_ctx* ctx, int32_t R, bool* ready) {
     *ready = false;
@@ -784,9 +784,11 @@ int t32_prepare(veloxq_ctx* ctx, int32_t R, bool* ready) {
         if (fused) room(ctx->s3[1], ob);
         room(ctx->dpart, pb);
         room(ctx->tcdone, db);
-        if (st == VELOXQ_ENOMEM) {        // no room: the SGEMM serves this context
+        if (st == VELOXQ_ENOMEM) {        // no room: the SGEMM serves this call, and has what these would hold
             ctx->q3.release();
-            ctx->q3_state = -1;
+            ctx->s3[0].release();
+            ctx->s3[1].release();
+            ctx->q3_state = 0;
             return VELOXQ_OK;
         }
         VQ_TRY(st);
