@@ -771,8 +771,19 @@ int veloxq_solve(veloxq_ctx* ctx, int32_t replicas, int32_t steps, const veloxq_
         VQ_TRY(ctx->y.ensure(sizeof(float) * n * R));
         VQ_TRY(ctx->ework.ensure(sizeof(int64_t) * (size_t)nparts * R));
         VQ_TRY(ctx->flags.ensure((size_t)R));
-        if (path == VELOXQ_PATH_STREAM)
-            VQ_TRY(stream_autotune(ctx, replicas, ctx->s_a.as<float>(), ctx->s_b.as<float>(), ctx->y.as<float>()));
+        if (path == VELOXQ_PATH_STREAM) {
+            // runs of steps up to a readout that go by windows of replicas, and those that do not
+            bool by[2] = {false, false};
+            for (int k = 0, from = 0; k < steps; ++k)
+                if (is_readout(p, k)) {
+                    by[!std::getenv("VELOXQ_STREAM_FORM") && stream_window(ctx, replicas, k + 1 - from) != 0] = true;
+                    from = k + 1;
+                }
+            for (int w = 0; w < 2; ++w)
+                if (by[w])
+                    VQ_TRY(stream_autotune(ctx, replicas, ctx->s_a.as<float>(), ctx->s_b.as<float>(), ctx->y.as<float>(),
+                                           w != 0));
+        }
         TcRun tc;
         const bool use_tc = path == VELOXQ_PATH_DENSE && p.prec != VELOXQ_PREC_FP32;
         if (use_tc) VQ_TRY(tc_setup(ctx, p.prec, replicas, &tc, p.method));
@@ -893,7 +904,7 @@ int veloxq_solve(veloxq_ctx* ctx, int32_t replicas, int32_t steps, const veloxq_
         ex->timing.path = (int32_t)path;
         ex->timing.main_launches = main_launches;
         const bool streamed = path == VELOXQ_PATH_STREAM;
-        ex->timing.stream_gather = streamed ? ctx->stream_unroll : 0;
+        ex->timing.stream_gather = streamed ? (window ? ctx->stream_wunroll : ctx->stream_unroll) : 0;
         ex->timing.stream_chunk = streamed ? (window ? window : ctx->stream_cvec * vec_width(replicas)) : 0;
         ex->timing.batch_stages = 0;
         ex->timing.batch_group = 0;
@@ -1299,7 +1310,7 @@ int veloxq_grad(veloxq_ctx* ctx, int32_t replicas, int32_t steps, const veloxq_s
         DevBuf t;
         VQ_TRY(t.ensure(3 * blk));
         VQ_TRY(stream_autotune(ctx, replicas, t.as<float>(), t.as<float>() + ctx->n * (int64_t)replicas,
-                               t.as<float>() + 2 * ctx->n * (int64_t)replicas));
+                               t.as<float>() + 2 * ctx->n * (int64_t)replicas, false));
     }
     double dc0 = 0.0;
     AdjTiming tm;

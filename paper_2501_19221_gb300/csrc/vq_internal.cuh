@@ -163,6 +163,8 @@ struct veloxq_ctx {
                                   // 6 couplings); 0: not tuned yet
     int32_t stream_tuned_R = -1;  // replica count the variant was tuned for
     int32_t stream_cvec = 0;      // replica vectors per chunk of the streaming step's thread order (0: all)
+    int stream_wunroll = 0;       // gather variant of steps of one window of replicas
+    int32_t stream_wtuned_R = -1;
 };
 
 namespace vq {
@@ -224,7 +226,7 @@ int stream_step_y(veloxq_ctx* ctx, int32_t R, const float* S_cur, float* S_nxt, 
                   const float* a_table, int k, float dt, float a0, float c0, float* F_out,
                   const Rule& rule = Rule());
 int vec_width(int32_t R);
-int stream_autotune(veloxq_ctx* ctx, int32_t R, float* S_a, float* S_b, float* Y);
+int stream_autotune(veloxq_ctx* ctx, int32_t R, float* S_a, float* S_b, float* Y, bool windows);
 
 // sparse resident kernel (vq_resident.cu)
 bool resident_fits(const veloxq_ctx* ctx, int32_t R, int* rc, int* threads, size_t* smem);

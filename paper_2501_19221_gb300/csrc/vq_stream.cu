@@ -294,8 +294,9 @@ int launch_step(veloxq_ctx* ctx, int32_t R, const float* S_cur, float* S_nxt, co
     } while (0)
     // without a timing trial (single steps and fields): six at once on rows of exactly six couplings, where it is
     // the form every trial picks (cubic lattice L = 100, 256 replicas: 0.70 ms against 0.80 one at a time)
-    const bool six = ctx->uniform_deg == 6 && (ctx->stream_unroll == 6 || ctx->stream_unroll == 0);
-    const int unroll = six ? 6 : ctx->stream_unroll == 4 ? 4 : 1;
+    const int form = rn ? ctx->stream_wunroll : ctx->stream_unroll;
+    const bool six = ctx->uniform_deg == 6 && (form == 6 || form == 0);
+    const int unroll = six ? 6 : form == 4 ? 4 : 1;
     if (ctx->w8.p) {
         const int8_t* w = ctx->w8.as<int8_t>();
         if (V == 4) VQ_STEP(4, int8_t, w, 0.5f); else if (V == 2) VQ_STEP(2, int8_t, w, 0.5f); else VQ_STEP(1, int8_t, w, 0.5f);
@@ -383,10 +384,14 @@ static std::vector<int32_t> chunk_candidates(int64_t n, int32_t R) {
 // Pick the gather variant (one, four or six couplings at a time) and the
 // replica chunk width of the streaming kernels for R replicas by timing steps
 // of each pair on the caller's buffers (contents are overwritten);
-// VELOXQ_STREAM_FORM fixes them instead.
+// VELOXQ_STREAM_FORM fixes them instead. windows: for runs by windows of
+// replicas, whose gather is picked on steps of one window; steps over all
+// replicas (the caller's own steps on this context) then keep this gather with
+// the chunk width that suits them, until a call that runs such steps itself
+// tries every pair.
 // Runs eagerly on ctx->stream; must not be called during stream capture.
-int stream_autotune(veloxq_ctx* ctx, int32_t R, float* S_a, float* S_b, float* Y) {
-    if (ctx->stream_unroll != 0 && ctx->stream_tuned_R == R) return VELOXQ_OK;
+int stream_autotune(veloxq_ctx* ctx, int32_t R, float* S_a, float* S_b, float* Y, bool windows) {
+    if ((windows ? ctx->stream_wtuned_R : ctx->stream_tuned_R) == R) return VELOXQ_OK;
     if (const char* form = std::getenv("VELOXQ_STREAM_FORM")) {
         // a form fixed by the caller: "gather chunk", the chunk in replicas (0: all at once)
         const int V = vec_width(R);
@@ -400,9 +405,9 @@ int stream_autotune(veloxq_ctx* ctx, int32_t R, float* S_a, float* S_b, float* Y
             return fail(VELOXQ_EINVAL, "VELOXQ_STREAM_FORM must be \"gather chunk\": gather 1, 4 or 6 (rows of exactly "
                                        "6 couplings) and a chunk of replicas (0: all) that the replica count splits "
                                        "into");
-        ctx->stream_unroll = u;
+        ctx->stream_unroll = ctx->stream_wunroll = u;
         ctx->stream_cvec = cv;
-        ctx->stream_tuned_R = R;
+        ctx->stream_tuned_R = ctx->stream_wtuned_R = R;
         return VELOXQ_OK;
     }
     cudaEvent_t e0, e1;
@@ -410,49 +415,74 @@ int stream_autotune(veloxq_ctx* ctx, int32_t R, float* S_a, float* S_b, float* Y
     VQ_CUDA(cudaEventCreate(&e1));
     VQ_TRY(launch_init_state(ctx, R, 1, 0.1f, LAYOUT_NR, S_a, Y));
     const float* at = ctx->a_table.as<float>();
-    std::vector<std::pair<int, int32_t>> cands;   // (gather, chunk)
-    const int32_t win = stream_window(ctx, R, 50);  // runs by windows: their steps are timed, without chunks
-    for (int32_t cv : win ? std::vector<int32_t>{0} : chunk_candidates(ctx->n, R))
-        for (int u : {1, 4, 6})
-            if (u != 6 || ctx->uniform_deg == 6) cands.emplace_back(u, cv);
-    auto timed = [&](int reps, float* ms) -> int {
+    const int32_t win = windows ? stream_window(ctx, R, 50) : 0;
+    auto timed = [&](int reps, int32_t rn, float* ms) -> int {
         VQ_CUDA(cudaEventRecord(e0, ctx->stream));
         for (int k = 0; k < reps; ++k)
             VQ_TRY((launch_step<false, false>(ctx, R, (k & 1) ? S_b : S_a, (k & 1) ? S_a : S_b, Y, Y, at, 0, 0.5f,
-                                              1.0f, 0.1f, nullptr, Rule(), 0, win)));
+                                              1.0f, 0.1f, nullptr, Rule(), 0, rn)));
         VQ_CUDA(cudaEventRecord(e1, ctx->stream));
         VQ_CUDA(cudaEventSynchronize(e1));
         VQ_CUDA(cudaEventElapsedTime(ms, e0, e1));
         return VELOXQ_OK;
     };
-    // Two rounds over all candidates, each timing `reps` steps of one form
-    // (10 when a step is shorter than 0.3 ms, else 3); a form's time is its
+    // Two rounds over all candidates (gather, chunk), each timing `reps` steps of one form
+    // (`most`, 10 for the call's own steps, when a step is shorter than 0.3 ms, else 3); a form's time is its
     // faster round, so a round disturbed by the previous form's state in L2
     // or by a clock change does not decide the pick.
-    std::vector<float> per_step(cands.size(), 1e30f);
-    int reps = 3;
-    for (int round = 0; round < 2; ++round)
-        for (size_t c = 0; c < cands.size(); ++c) {
-            ctx->stream_unroll = cands[c].first;
-            ctx->stream_cvec = cands[c].second;
-            float ms = 0.f;
-            if (round == 0) {
-                VQ_TRY(timed(1, &ms));                 // warm; the first form's step sets the step count
-                if (c == 0 && ms < 0.3f) reps = 10;
+    auto pick = [&](const std::vector<std::pair<int, int32_t>>& cands, int32_t rn, int most, size_t* best) -> int {
+        std::vector<float> per_step(cands.size(), 1e30f);
+        int reps = 3;
+        for (int round = 0; round < 2; ++round)
+            for (size_t c = 0; c < cands.size(); ++c) {
+                ctx->stream_unroll = ctx->stream_wunroll = cands[c].first;
+                ctx->stream_cvec = cands[c].second;
+                float ms = 0.f;
+                if (round == 0) {
+                    VQ_TRY(timed(1, rn, &ms));             // warm; the first form's step sets the step count
+                    if (c == 0 && ms < 0.3f) reps = most;
+                }
+                VQ_TRY(timed(reps, rn, &ms));
+                per_step[c] = std::min(per_step[c], ms / (float)reps);
             }
-            VQ_TRY(timed(reps, &ms));
-            per_step[c] = std::min(per_step[c], ms / (float)reps);
-        }
+        *best = 0;
+        for (size_t c = 1; c < cands.size(); ++c)
+            if (per_step[c] < per_step[*best]) *best = c;
+        return VELOXQ_OK;
+    };
+    const int keep_u = ctx->stream_unroll, keep_w = ctx->stream_wunroll;
+    const int32_t keep_cv = ctx->stream_cvec;
+    std::vector<std::pair<int, int32_t>> cands;
+    for (int32_t cv : win ? std::vector<int32_t>{0} : chunk_candidates(ctx->n, R))
+        for (int u : {1, 4, 6})
+            if (u != 6 || ctx->uniform_deg == 6) cands.emplace_back(u, cv);
+    size_t bi = 0;
+    VQ_TRY(pick(cands, win, 10, &bi));
+    const int u = cands[bi].first;
+    if (!windows) {
+        ctx->stream_unroll = u;
+        ctx->stream_cvec = cands[bi].second;
+        ctx->stream_tuned_R = R;
+        ctx->stream_wunroll = keep_w;
+    } else if (ctx->stream_tuned_R == R) {
+        ctx->stream_unroll = keep_u;
+        ctx->stream_cvec = keep_cv;
+    } else {
+        const std::vector<int32_t> chunks = chunk_candidates(ctx->n, R);
+        std::vector<std::pair<int, int32_t>> whole;
+        for (int32_t cv : chunks) whole.emplace_back(u, cv);
+        bi = 0;
+        if (whole.size() > 1) VQ_TRY(pick(whole, 0, 3, &bi));   // no steps of this call: 3 at most
+        ctx->stream_unroll = u;
+        ctx->stream_cvec = whole[bi].second;
+        ctx->stream_tuned_R = -1;
+    }
+    if (windows) {
+        ctx->stream_wunroll = u;
+        ctx->stream_wtuned_R = R;
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    size_t bi = 0;
-    for (size_t c = 1; c < cands.size(); ++c)
-        if (per_step[c] < per_step[bi]) bi = c;
-    const int pick = cands[bi].first;
-    const int32_t pick_cv = cands[bi].second;
-    ctx->stream_unroll = pick;
-    ctx->stream_cvec = pick_cv;
-    ctx->stream_tuned_R = R;
     return VELOXQ_OK;
 }
 
