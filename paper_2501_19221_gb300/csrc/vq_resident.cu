@@ -69,7 +69,7 @@ ResPlan make_plan(const veloxq_ctx* ctx, int32_t R) {
             if (cs >= 1 && !csr_smem) continue;
             if (cs == 2 && !ell) continue;
             const SmemPlan p = plan_smem(n, csr_smem ? ctx->nnz : 0, rc, threads, nwords, csr_smem, csr_smem && packed,
-                                         ell ? ell_d : 0);
+                                         ell ? ell_d : 0, ell && rc <= 2 && row_in_registers(rpt, ell_d, threads));
             if (p.total > (size_t)kSmemMax) continue;
             const int64_t ctas = div_up(R, rc);
             const double cost = (double)div_up(ctas, sms) * (3.0 + rc) * (csr_smem ? 1.0 : 1.3);

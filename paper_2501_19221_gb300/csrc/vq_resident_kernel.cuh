@@ -129,13 +129,15 @@ struct SmemPlan {
 
 __host__ __device__ inline size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
 
+// zeros: one 128-byte line of zeros behind the rows, which slots past a row's
+// count read in the form that keeps its couplings unpacked (small instances;
+// the others, which may fill shared memory, have none)
 __host__ __device__ inline SmemPlan plan_smem(int n, int64_t nnz, int RC, int threads, int nwords, bool csr_smem,
-                                              bool packed, int ell_d) {
+                                              bool packed, int ell_d, bool zeros) {
     SmemPlan p;
     size_t o = 0;
-    // whole 128-byte lines (swizzle); in the ELL layouts one line of zeros behind them, which slots past a
-    // row's count read where the slot loop runs in whole groups
-    const size_t rows = (size_t)((n * RC + 31) / 32 * 32) + (ell_d > 0 ? 32 : 0);
+    // whole 128-byte lines (swizzle)
+    const size_t rows = (size_t)((n * RC + 31) / 32 * 32) + (zeros ? 32 : 0);
     p.s0 = o; o = align16(o + sizeof(float) * rows);
     p.s1 = o; o = align16(o + sizeof(float) * rows);
     p.b = o; o = align16(o + sizeof(float) * (size_t)n);
@@ -230,7 +232,9 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(const ResArgs a) {
     const int tid = threadIdx.x;
     const int lane = tid & 31, warp = tid >> 5;
     const int r0 = blockIdx.x * RC;
-    const SmemPlan pl = plan_smem(n, CSR_SMEM ? a.rowptr[n] : 0, RC, T, a.nwords, CSR_SMEM, PACKED, ELL ? a.ell_d : 0);
+    // ELL == 32 with one or two replicas: the couplings unpacked in registers (below)
+    constexpr bool OWN = ELL == 32 && RC <= 2;
+    const SmemPlan pl = plan_smem(n, CSR_SMEM ? a.rowptr[n] : 0, RC, T, a.nwords, CSR_SMEM, PACKED, ELL ? a.ell_d : 0, OWN);
     float* sA = reinterpret_cast<float*>(smem + pl.s0);
     float* sB = reinterpret_cast<float*>(smem + pl.s1);
     float* bsh = reinterpret_cast<float*>(smem + pl.b);
@@ -271,7 +275,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(const ResArgs a) {
     }
     for (int w = tid; w < RC * a.nwords; w += T) bits[w] = 0u;
     if (tid < RC) best[tid] = INT64_MAX;
-    if constexpr (ELL != 0) {
+    if constexpr (OWN) {
         // the line of zeros: behind the rows of both state buffers and (PA) of both spin buffers
         if (tid < 32) {
             const int z = (n * RC + 31) / 32 * 32 + tid;
@@ -328,7 +332,6 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(const ResArgs a) {
     // with the thread's own state and bias beside them, since a step of one
     // or two warps is a chain of latencies; with more replicas, whose registers
     // do not suffice for that, as the coupling words.
-    constexpr bool OWN = ELL == 32 && RC <= 2;
     uint32_t pk[ELL == 32 && !OWN ? 32 : 1];
     float pw[OWN ? 32 : 1];
     int po[OWN ? 32 : 1];
@@ -682,6 +685,10 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(const ResArgs a) {
 
 using KFn = void (*)(const ResArgs);
 
+// ELL layout with one row per thread and at most 32 slots: the coupling words
+// in registers, which takes the 128-register budget of a 512-thread CTA
+inline bool row_in_registers(int rpt, int ell_d, int threads) { return rpt == 1 && ell_d > 0 && ell_d <= 32 && threads <= 512; }
+
 // 1024-thread CTAs keep at most 8 momenta per thread in registers (64-register
 // cap); 512-thread CTAs up to 32.
 template <int RC, int RPT, int METHOD> KFn pick_csr(bool csr_smem, bool packed, int ell_d, int threads) {
@@ -691,8 +698,7 @@ template <int RC, int RPT, int METHOD> KFn pick_csr(bool csr_smem, bool packed, 
     } else {
         if (!csr_smem) return k_resident<RC, RPT, false, false, MAXT, 0, METHOD>;
         if constexpr (RPT == 1) {
-            // the 32 coupling words need the 128-register budget of a 512-thread CTA
-            if (ell_d > 0 && ell_d <= 32 && threads <= 512) return k_resident<RC, 1, true, true, 512, 32, METHOD>;
+            if (row_in_registers(RPT, ell_d, threads)) return k_resident<RC, 1, true, true, 512, 32, METHOD>;
         }
         if (ell_d == 6) return k_resident<RC, RPT, true, true, MAXT, 6, METHOD>;
         if (ell_d > 0) return k_resident<RC, RPT, true, true, MAXT, 1, METHOD>;
