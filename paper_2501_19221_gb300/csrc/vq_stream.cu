@@ -265,12 +265,22 @@ int launch_step(veloxq_ctx* ctx, int32_t R, const float* S_cur, float* S_nxt, co
     const int64_t total = ctx->n * (int64_t)nvec;
     const unsigned g = (unsigned)div_up(total, 256);
     // Short steps are launched dependently, so that a step's launch and first
-    // blocks overlap the last ones of the step before: Pegasus P_16 at 128 /
-    // 1024 replicas 6.0 -> 4.7 / 27.8 -> 27.4 us per step, Zephyr Z_12 at 1024
-    // 28.6 -> 26.8. Longer steps lose by it (3R3X at 256 replicas 237 -> 248 us,
-    // lattice L = 100 677 -> 715: blocks of two steps share L2).
+    // blocks overlap the last ones of the step before. Plain -> dependent, us
+    // per step, by threads per step: tile planting L = 100 0.16 / 1.28 M 3.3 ->
+    // 2.6 / 12.6 -> 12.1; lattice L = 40 0.26 / 1.28 / 1.54 / 3.1 M 4.0 -> 3.8 /
+    // 12.0 -> 11.5 / 14.0 -> 14.2 / 36.4 -> 37.1; 3R3X (2e4 variables) 0.64 /
+    // 1.28 / 2.6 M 9.3 -> 8.9 / 16.5 -> 16.6 / 40.0 -> 42.8; Pegasus P_16 1.44 /
+    // 2.9 M 27.7 -> 27.2 / 63.4 -> 60.7; the longest steps lose (3R3X at 256
+    // replicas 237 -> 248, lattice L = 100 677 -> 715: blocks of two steps
+    // share L2), most from 1.5 M threads on.
+    // Rows of unequal length of many variables with few replicas lose at any
+    // size: 3-body chain (2e5 variables) at 1 / 16 replicas 3.3 -> 3.7 / 10.9
+    // -> 11.4, 3R3X (2e5) at 4 8.3 -> 9.4, Zephyr Z_40 (51840) at 16 8.9 -> 9.4;
+    // with 2e4 variables or 64 replicas they gain (chain 4.3 -> 3.6, Pegasus
+    // P_30 at 16 4.6 -> 4.1, Z_40 at 64 20.7 -> 19.9).
     // A field alone has no step before it to overlap.
-    const bool dependent = !FIELD_ONLY && total <= 1500000;
+    const bool scattered = ctx->uniform_deg < 0 && ctx->n > 40000 && nvec <= 4;
+    const bool dependent = !FIELD_ONLY && total <= 1500000 && !scattered;
     const int64_t* rp = ctx->rowptr.as<int64_t>();
     const int32_t* cl = ctx->col.as<int32_t>();
     const float* bf = ctx->bf.as<float>();
@@ -327,9 +337,13 @@ int stream_step(veloxq_ctx* ctx, int32_t R, const float* S_cur, float* S_nxt, fl
 // replicas after the other. When the state of all replicas lies well beyond
 // L2 but a window's two state arrays and momenta stay in it with the
 // couplings, every step after a window's first reads and writes L2 instead
-// of HBM. The widest window of at most 96 MB is taken (L2 holds 126 MB), of at
-// least 32 replicas (one 128-byte line per row) and 2.5 M variable-replicas
-// (shorter steps cost more in launches than they save).
+// of HBM. The widest window of at most 96 MB is taken (L2 holds 126 MB; tile
+// planting L = 300 at 256 replicas, 65.6 us all at once: windows of 35 / 69 /
+// 138 MB 63.2 / 59.2 / 72.2 us; 3R3X of 3e5 variables, window 127 MB: 377
+// either way), of at least 32 replicas (one 128-byte line per row) and 2.5 M
+// variable-replicas (shorter steps cost more in launches than they save:
+// lattices of 1.6 / 2.4 / 3.1 M per window 51.5 -> 56.7, 72.5 -> 73.6, 61.6 ->
+// 56.8 us; random graphs would gain below too, 3R3X 1.9 M 95 -> 83).
 int32_t stream_window(const veloxq_ctx* ctx, int32_t R, int steps) {
     const double l2 = 126e6, room = 96e6;
     const double couplings = (double)ctx->nnz * (ctx->w8.p ? 5.0 : 8.0) + 12.0 * (double)ctx->n;
