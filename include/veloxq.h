@@ -95,8 +95,8 @@ typedef enum { VELOXQ_I8 = 0, VELOXQ_I32 = 1, VELOXQ_F32 = 2, VELOXQ_F64 = 3 } v
  *                  normwise). Parallel Annealing's operand (+-1) is exact in one
  *                  term, so FP8 runs it this way too.
  * BF16 and FP8 run every step up to a readout in one persistent launch; its
- * tiles go column block (256 replicas) by column block, in groups of two
- * blocks for BF16 and FP8_ONE_TERM. The environment variable
+ * tiles go column block (256, 128 or 64 replicas, by n and R) by column block,
+ * in groups of two blocks for BF16 and FP8_ONE_TERM. The environment variable
  * VELOXQ_TC_COLGROUP (1 to 16 blocks per group) fixes the group; the results
  * are the same bits for every group. */
 typedef enum {

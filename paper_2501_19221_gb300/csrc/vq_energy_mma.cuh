@@ -16,17 +16,22 @@
 // added, shifted by 12 k, into 64-bit totals modulo 2^64, which is exact
 // because the finished energy lies in range.
 //
-// What bounds it: instruction issue (digit extraction, fragment loads, the
-// masked integer sums), not memory. The previous form selected and added
-// int64 couplings on the CUDA cores, four instructions per coupling and
+// What bounds it: latency, not memory and not a pipe. One block of 16 warps
+// fits per SM (124 registers for 512 threads): four warps per scheduler, which
+// issue in 44 % of the cycles (n = 2048, 1024 vectors, int32 couplings; the
+// tensor pipe 10 %) and otherwise wait on fixed latencies, the loads of the
+// next stage, the fragments from shared memory and the barrier behind every
+// digit plane; the 256 blocks are 1.7 waves on 152 SMs. Every block of 128
+// vectors cuts its tile of Q into digits anew. The previous form selected and
+// added int64 couplings on the CUDA cores, four instructions per coupling and
 // replica; here a coupling costs a few per digit for all replicas of the
-// tile. Measured at n = 2048, 1024 vectors, int32 couplings (one digit):
-// 957 -> 126 us; the readout of 256 Wishart instances (n 100 to 2000, 64
-// replicas, FP32 couplings, four digits): 12.3 -> 4 ms. The products go
-// through mma.sync rather than tcgen05 because
-// this kernel serves calls that neither synchronise nor allocate
-// (veloxq_energy_dev and its no-allocation form), where no bounded
-// tensor-memory wait could be reported and no digit planes can be kept.
+// tile. Measured at n = 2048, 1024 vectors: int32 and int8 couplings (one
+// digit) 957 -> 136 us, FP32 couplings 279 us; the readout of 256 Wishart instances (n 100 to 2000, 64 replicas, FP32
+// couplings, four digits): 12.3 -> 2.3 ms. The products go through mma.sync
+// because a tile's digits are cut in registers and go to shared memory at
+// once: tcgen05 would take 256 x 128 tiles, hence planes kept in memory, and
+// this kernel serves calls that must not allocate (veloxq_energy_dev and its
+// no-allocation form).
 #pragma once
 
 #include <cuda_fp16.h>
