@@ -824,6 +824,10 @@ int t32_split(veloxq_ctx* ctx, int32_t R, const float* S, const Rule& rule, bool
         t->seq = ctx->t32_seq;
         bad = ctx->t32w.as<uint32_t>() + 1;
         bad_h = reinterpret_cast<uint32_t*>(ctx->t32h.dev) + 1;
+        // a captured call is replayed with its number: what an earlier replay found must not stay
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        VQ_CUDA(cudaStreamIsCapturing(ctx->stream, &cs));
+        if (cs != cudaStreamCaptureStatusNone) VQ_CUDA(cudaMemsetAsync(bad, 0, sizeof(uint32_t), ctx->stream));
     }
     t->terms = rule.method == VELOXQ_METHOD_PA ? 1 : 3;
     // the other operand buffer, which the epilogue writes first: its K padding must be zero too

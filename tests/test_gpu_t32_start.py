@@ -62,3 +62,34 @@ def test_state_that_overflows_within_a_call(B, n, R):
     keep = torch.arange(R, device="cuda") != 3
     assert bool(torch.isfinite(a[keep]).all())
     assert float((a[keep] - b[keep]).norm() / b[keep].norm()) <= 1e-5
+
+
+def test_replays_of_a_captured_field_are_checked_one_by_one(B):
+    """A replay whose state is outside the terms' range is served by the FP32 sums; the next replay with an ordinary
+    state gives the tensor cores' bits again."""
+    n, R = 600, 40
+    J, _ = I.sk_qubo(n, seed=0)
+    ctx = B.veloxq_create_ising_dense(J)
+    g = torch.Generator(device="cuda").manual_seed(1)
+    S0 = torch.rand(R, n, generator=g, device="cuda") * 2 - 1
+    S, F = S0.clone(), torch.empty_like(S0)
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        B.veloxq_field_dev(ctx, R, B.VELOXQ_PREC_FP32, S, F)
+        side.synchronize()
+        want = F.clone()
+        graph = torch.cuda.CUDAGraph()
+        graph.capture_begin()
+        B.veloxq_field_dev(ctx, R, B.VELOXQ_PREC_FP32, S, F)
+        graph.capture_end()
+        for value in (None, float("inf"), None):
+            S.copy_(S0)
+            if value is not None:
+                S[2, 7] = value
+            F.zero_()
+            graph.replay()
+            side.synchronize()
+            if value is None:
+                assert torch.equal(F, want)
+            else:
+                assert bool(torch.isinf(F[2]).any()) and bool(torch.isfinite(F[3]).all())
