@@ -1,46 +1,59 @@
 """FP32 fields of a dense context while device memory is short: a call for
 whose terms there is no room runs as FP32 sums of products, and later calls
-run on the tensor cores again."""
+run on the tensor cores again. In a process of its own: the library's cache of
+freed buffers would otherwise serve the call from what earlier tests left."""
+import os
+import subprocess
+import sys
+
 import pytest
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
-@pytest.fixture(scope="module")
-def B():
+_CHILD = """
+import sys
+sys.path.insert(0, sys.argv[1])
+import torch
+from paper_2501_19221_gb300 import binding as B
+
+n, few, many = 4096, 64, 20000
+g = torch.Generator(device="cuda").manual_seed(0)
+Q = torch.randn(n, n, generator=g, device="cuda").triu_(1)
+Q = (Q + Q.T) / n ** 0.5
+ctx = B.veloxq_create_dense(Q.cpu().numpy())
+S = torch.rand(many, n, generator=g, device="cuda") * 2 - 1
+F = torch.empty_like(S)
+
+def field(R):
+    F[:R] = 0
+    B.veloxq_field_dev(ctx, R, B.VELOXQ_PREC_FP32, S[:R], F[:R])
+    torch.cuda.synchronize()
+    ref = S[:few].double() @ Q.double()
+    return F[:few].clone(), float((F[:few].double() - ref).norm() / ref.norm())
+
+want, e = field(few)
+assert e <= 2e-7, e                            # tensor cores (9e-8); the FP32 sums have 6e-7 at this size
+torch.cuda.empty_cache()
+free, _ = torch.cuda.mem_get_info()
+hold = torch.empty(max(0, free - (300 << 20)), dtype=torch.uint8, device="cuda")     # 300 MB left; terms: 491 MB
+_, e = field(many)
+assert 2e-7 < e <= 2e-6, e
+del hold
+torch.cuda.empty_cache()
+got, _ = field(few)
+assert torch.equal(got, want)
+print("ok")
+"""
+
+
+def test_no_room_for_one_call():
     if not torch.cuda.is_available():
         pytest.skip("needs a CUDA device")
     import __graft_entry__ as g
     g.build()
-    from paper_2501_19221_gb300 import binding
-    return binding
-
-
-def test_no_room_for_one_call(B):
-    n, few, many = 4096, 64, 20000
-    g = torch.Generator(device="cuda").manual_seed(0)
-    Q = torch.randn(n, n, generator=g, device="cuda").triu_(1)
-    Q = (Q + Q.T) / n ** 0.5
-    ctx = B.veloxq_create_dense(Q.cpu().numpy())
-    S = torch.rand(many, n, generator=g, device="cuda") * 2 - 1
-    F = torch.empty_like(S)
-
-    def field(R):
-        F[:R] = 0
-        B.veloxq_field_dev(ctx, R, B.VELOXQ_PREC_FP32, S[:R], F[:R])
-        torch.cuda.synchronize()
-        ref = S[:few].double() @ Q.double()
-        return F[:few].clone(), float((F[:few].double() - ref).norm() / ref.norm())
-
-    want, e = field(few)
-    assert e <= 2e-7                               # tensor cores (9e-8); the FP32 sums have 6e-7 at this size
     torch.cuda.empty_cache()
-    free, _ = torch.cuda.mem_get_info()
-    hold = torch.empty(max(0, free - (300 << 20)), dtype=torch.uint8, device="cuda")     # 300 MB left; terms: 491 MB
-    _, e = field(many)
-    assert 2e-7 < e <= 2e-6
-    del hold
-    torch.cuda.empty_cache()
-    got, _ = field(few)
-    assert torch.equal(got, want)
+    r = subprocess.run([sys.executable, "-c", _CHILD, ROOT], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and r.stdout.strip().endswith("ok"), r.stdout + r.stderr
