@@ -441,12 +441,12 @@ int stream_autotune(veloxq_ctx* ctx, int32_t R, float* S_a, float* S_b, float* Y
         return VELOXQ_OK;
     };
     // Two rounds over all candidates (gather, chunk), each timing `reps` steps of one form
-    // (`most`, 10 for the call's own steps, when a step is shorter than 0.3 ms, else 3); a form's time is its
+    // (`most`, 10 for the call's own steps, when a step is shorter than 0.3 ms, else at most 3); a form's time is its
     // faster round, so a round disturbed by the previous form's state in L2
     // or by a clock change does not decide the pick.
     auto pick = [&](const std::vector<std::pair<int, int32_t>>& cands, int32_t rn, int most, size_t* best) -> int {
         std::vector<float> per_step(cands.size(), 1e30f);
-        int reps = 3;
+        int reps = std::min(3, most);
         for (int round = 0; round < 2; ++round)
             for (size_t c = 0; c < cands.size(); ++c) {
                 ctx->stream_unroll = ctx->stream_wunroll = cands[c].first;
@@ -486,7 +486,7 @@ int stream_autotune(veloxq_ctx* ctx, int32_t R, float* S_a, float* S_b, float* Y
         std::vector<std::pair<int, int32_t>> whole;
         for (int32_t cv : chunks) whole.emplace_back(u, cv);
         bi = 0;
-        if (whole.size() > 1) VQ_TRY(pick(whole, 0, 3, &bi));   // no steps of this call: 3 at most
+        if (whole.size() > 1) VQ_TRY(pick(whole, 0, 1, &bi));   // no steps of this call: one each
         ctx->stream_unroll = u;
         ctx->stream_cvec = whole[bi].second;
         ctx->stream_tuned_R = -1;
