@@ -41,9 +41,10 @@
 // replicas), M = 256 MMAs issued by the even CTA, operands staged by TMA in
 // blocks of 64 variables: the three terms of a CTA's 128 rows (48 KB) and of
 // its 64 replicas (24 KB) in one 3-D copy each, 3 stages (blocks of 32, whose
-// rows are half as long, took 631 instead of 585 us at n = 8192). Tiles of 128
-// replicas rather than 256 keep a thread's part of the drained field in 64
-// registers, and give twice the tiles to spread over the SMs.
+// rows are half as long, took 631 instead of 585 us at n = 8192, with six
+// products). Tiles of 128 replicas rather than 256 keep a thread's two parts of
+// the drained field in 128 registers, and give twice the tiles to spread over
+// the SMs.
 //   * Enough tiles (more than half of the pairs): one launch runs every step
 //     up to a readout, tiles of consecutive steps overlapping as in vq_tc.cu
 //     (and one behind it that only works where SMs were held by others).
