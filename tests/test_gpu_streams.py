@@ -111,6 +111,24 @@ def _held_steps(ctx, B, stream, R, S, Y, sched):
         return stream.record_event()
 
 
+@pytest.mark.parametrize("default_first", [True, False])
+def test_default_stream_and_another(B, default_first):
+    """The legacy default stream orders itself only behind streams that ask for it; these do not."""
+    ctx, n = _dense(B, 300)
+    R, sched = 17, B.make_schedule(c0=1.0)
+    states = [_state(R, n, s) for s in (1, 2)]
+    B.veloxq_steps_dev(ctx, R, 0, 1, 20, sched, *_state(R, n, 1))
+    torch.cuda.synchronize()
+    pair = [torch.cuda.default_stream(), torch.cuda.Stream()]
+    first, second = pair if default_first else pair[::-1]
+    e1 = _held_steps(ctx, B, first, R, *states[0], sched)
+    with torch.cuda.stream(second):
+        B.veloxq_steps_dev(ctx, R, 0, 1, 20, sched, *states[1])
+        e2 = second.record_event()
+    e2.synchronize()
+    assert e1.query()
+
+
 def test_third_stream_waits_too(B):
     """A call in between that leaves nothing on the scratch does not end the wait for the first one."""
     ctx, n = _dense(B, 300)
